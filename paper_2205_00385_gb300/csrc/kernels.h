@@ -161,7 +161,10 @@ long long stencil_values(int dim, int t, const GridP& g);
 // (float64); y = A x with A float64 and x, y of storage t
 cudaError_t launch_dense_assemble(int dim, int t, int ta, const GridP& g, const uint8_t* mask,
                                   const void* Kc, void* A, double shift, cudaStream_t s);
-cudaError_t launch_cholesky_inverse(int t, int n, void* A, void* Ainv, int* status,
+// A is overwritten with L^{-1} (A = L L^T); scratch holds coarse_scratch_values(n)
+// values of type t; a non-positive pivot sets *status = TO_E_SINGULAR
+long long coarse_scratch_values(long long n);
+cudaError_t launch_cholesky_inverse(int t, int n, void* A, void* Ainv, void* scratch, int* status,
                                     cudaStream_t s);
 cudaError_t launch_dense_gemv(int ta, int t, int n, const void* A, const void* x, void* y,
                               cudaStream_t s);

@@ -321,240 +321,6 @@ __global__ void __launch_bounds__(256)
   A[t] = row == col ? (TA)((double)s * (1.0 + shift)) : s;
 }
 
-// In-place Cholesky (lower) of the n x n row-major matrix A by one block,
-// right-looking.  A non-positive pivot sets *status = TO_E_SINGULAR.
-template <typename T>
-__global__ void __launch_bounds__(1024) k_cholesky(int n, T* __restrict__ A, int* status) {
-  __shared__ int s_bad;
-  if (threadIdx.x == 0) s_bad = 0;
-  __syncthreads();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, nty = blockDim.x >> 5;
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) {
-      T d = A[(size_t)k * n + k];
-      if (!(d > T(0))) {
-        s_bad = 1;
-        d = T(1);
-      }
-      A[(size_t)k * n + k] = sqrt(d);
-    }
-    __syncthreads();
-    const T lkk = A[(size_t)k * n + k];
-    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) A[(size_t)i * n + k] /= lkk;
-    __syncthreads();
-    for (int i = k + 1 + ty; i < n; i += nty) {
-      const T lik = A[(size_t)i * n + k];
-      for (int j = k + 1 + tx; j <= i; j += 32) A[(size_t)i * n + j] -= lik * A[(size_t)j * n + k];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && s_bad) *status = TO_E_SINGULAR;
-}
-
-// Blocked right-looking Cholesky (lower, in place) by one block of 1024
-// threads: per 32-column block, the diagonal block is factored in shared
-// memory (one entry per thread in each column's update), the panel below it
-// is staged in shared memory and solved row by row, and the trailing lower
-// triangle is updated by all threads in 4 x 4 register tiles.
-constexpr int CB = 32, CBP = 33;
-
-__device__ __forceinline__ void tri_index(long long p, int& ii, int& jj) {
-  // float estimate (GB300's FP64 pipe is slow), corrected in integers
-  int r = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
-  while ((long long)r * (r + 1) / 2 > p) --r;
-  while ((long long)(r + 1) * (r + 2) / 2 <= p) ++r;
-  ii = r;
-  jj = (int)(p - (long long)r * (r + 1) / 2);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_cholesky_blocked(int n, T* __restrict__ A, int* status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* Dg = reinterpret_cast<T*>(smem_raw);   // CB x CBP
-  T* Pn = Dg + CB * CBP;                    // (n) x CBP panel rows
-  __shared__ int s_bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) s_bad = 0;
-  for (int k0 = 0; k0 < n; k0 += CB) {
-    const int kb = min(CB, n - k0);
-    for (int idx = tid; idx < kb * kb; idx += blockDim.x) {
-      const int r = idx / kb, cc = idx % kb;
-      Dg[r * CBP + cc] = A[(size_t)(k0 + r) * n + k0 + cc];
-    }
-    __syncthreads();
-    // diagonal block: per column j the pivot, the scaling of the column and
-    // the rank-1 update of the block's remaining lower triangle, one entry
-    // per thread (thread (r, cc) = (tid / 32, tid % 32))
-    {
-      const int r = tid >> 5, cc = tid & 31;
-      for (int j = 0; j < kb; ++j) {
-        if (tid == 0) {
-          T d = Dg[j * CBP + j];
-          if (!(d > T(0))) {
-            s_bad = 1;
-            d = T(1);
-          }
-          Dg[j * CBP + j] = sqrt(d);
-        }
-        __syncthreads();
-        if (tid > j && tid < kb) Dg[tid * CBP + j] /= Dg[j * CBP + j];
-        __syncthreads();
-        if (r > j && r < kb && cc > j && cc <= r) Dg[r * CBP + cc] -= Dg[r * CBP + j] * Dg[cc * CBP + j];
-        __syncthreads();
-      }
-    }
-    for (int idx = tid; idx < kb * kb; idx += blockDim.x) {
-      const int r = idx / kb, cc = idx % kb;
-      if (cc <= r) A[(size_t)(k0 + r) * n + k0 + cc] = Dg[r * CBP + cc];
-    }
-    const int m = n - k0 - kb;
-    // the panel below the diagonal block, staged by all threads (coalesced
-    // rows), then solved row by row in place
-    for (int idx = tid; idx < m * kb; idx += blockDim.x) {
-      const int r = idx / kb, cc = idx - r * kb;
-      Pn[r * CBP + cc] = A[(size_t)(k0 + kb + r) * n + k0 + cc];
-    }
-    __syncthreads();
-    for (int r = tid; r < m; r += blockDim.x) {
-      const size_t row = (size_t)(k0 + kb + r) * n + k0;
-      T xr[CB];
-#pragma unroll
-      for (int cc = 0; cc < CB; ++cc) {
-        if (cc < kb) {
-          T s = Pn[r * CBP + cc];
-#pragma unroll
-          for (int t = 0; t < CB; ++t)
-            if (t < cc) s -= xr[t] * Dg[cc * CBP + t];
-          xr[cc] = s / Dg[cc * CBP + cc];
-          A[row + cc] = xr[cc];
-          Pn[r * CBP + cc] = xr[cc];
-        }
-      }
-    }
-    __syncthreads();
-    // trailing update by 4 x 4 tiles of the lower triangle, one tile per
-    // thread and pass: each entry sums its kb products in the same order as
-    // an entry-wise loop, the tile's panel rows are read once per t
-    const int mt = (m + 3) >> 2;
-    const long long tiles = (long long)mt * (mt + 1) / 2;
-    for (long long p = tid; p < tiles; p += blockDim.x) {
-      int ti, tj;
-      tri_index(p, ti, tj);
-      const int r0 = 4 * ti, c0 = 4 * tj;
-      T acc[4][4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-      for (int t = 0; t < kb; ++t) {
-        T pr[4], pc[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          pr[a] = r0 + a < m ? Pn[(r0 + a) * CBP + t] : T(0);
-          pc[a] = c0 + a < m ? Pn[(c0 + a) * CBP + t] : T(0);
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] += pr[a] * pc[b];
-      }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int ii = r0 + a, jj = c0 + b;
-          if (ii < m && jj <= ii) A[(size_t)(k0 + kb + ii) * n + k0 + kb + jj] -= acc[a][b];
-        }
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && s_bad) *status = TO_E_SINGULAR;
-}
-
-// X = L^{-1} by forward substitution, one warp per column (stored in the
-// upper triangle-free buffer Linv, row-major, zero above the diagonal).
-template <typename T>
-__global__ void __launch_bounds__(256)
-    k_lower_inverse(int n, const T* __restrict__ L, T* __restrict__ X) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= n) return;
-  const int jc = warp;
-  for (int i = lane; i < jc; i += 32) X[(size_t)i * n + jc] = T(0);
-  if (lane == 0) X[(size_t)jc * n + jc] = T(1) / L[(size_t)jc * n + jc];
-  __syncwarp();
-  for (int i = jc + 1; i < n; ++i) {
-    T s = T(0);
-    for (int m = jc + lane; m < i; m += 32) s += L[(size_t)i * n + m] * X[(size_t)m * n + jc];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) X[(size_t)i * n + jc] = -s / L[(size_t)i * n + i];
-    __syncwarp();
-  }
-}
-
-// X = L^{-1} by column blocks: CTA jb owns the 32 columns jb*32 .. jb*32+31
-// of X (zero above row block jb) and walks the row blocks ib = jb, jb+1, ...
-// downwards: R = I(ib, jb) - sum_{kb < ib} L(ib, kb) X(kb, jb) (32 x 32
-// products, the L block staged in shared memory, the X column block kept
-// there), then one warp solves L(ib, ib) X(ib, jb) = R by forward
-// substitution, a column per lane.  1024 threads: (ty, tx) = (row, column)
-// within a block.
-template <typename T>
-__global__ void __launch_bounds__(1024) k_lower_inverse_blocked(int n, const T* __restrict__ L,
-                                                                T* __restrict__ X) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int nbk = (n + 31) / 32;
-  T* Xs = reinterpret_cast<T*>(smem_raw);   // [nbk * 32][32]
-  T* Ls = Xs + (size_t)nbk * 32 * 32;       // [32][33]
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int jb = blockIdx.x;
-  for (int ib = jb; ib < nbk; ++ib) {
-    T r = (ib == jb && ty == tx) ? T(1) : T(0);
-    const int lr = ib * 32 + ty;
-    for (int kb = jb; kb < ib; ++kb) {
-      const int lc = kb * 32 + tx;
-      Ls[ty * 33 + tx] = (lr < n && lc < n) ? L[(size_t)lr * n + lc] : T(0);
-      __syncthreads();
-#pragma unroll 8
-      for (int m = 0; m < 32; ++m) r -= Ls[ty * 33 + m] * Xs[(kb * 32 + m) * 32 + tx];
-      __syncthreads();
-    }
-    // diagonal block (identity beyond n, so padded rows solve to zero)
-    {
-      const int dc = ib * 32 + tx;
-      Ls[ty * 33 + tx] = (lr < n && dc < n) ? L[(size_t)lr * n + dc] : (ty == tx ? T(1) : T(0));
-    }
-    Xs[(ib * 32 + ty) * 32 + tx] = r;
-    __syncthreads();
-    if (ty == 0) {
-      T* xb = Xs + (size_t)ib * 32 * 32;
-      for (int k = 0; k < 32; ++k) {
-        T v = xb[k * 32 + tx];
-        for (int m = 0; m < k; ++m) v -= Ls[k * 33 + m] * xb[m * 32 + tx];
-        xb[k * 32 + tx] = v / Ls[k * 33 + k];
-      }
-    }
-    __syncthreads();
-  }
-  const int col = jb * 32 + tx;
-  if (col < n)
-    for (int row = ty; row < n; row += 32)
-      X[(size_t)row * n + col] = row >= jb * 32 ? Xs[row * 32 + tx] : T(0);
-}
-
-// Ainv = X^T X (X = L^{-1} lower triangular): Ainv[i][j] = sum_{m>=max(i,j)} X[m][i] X[m][j]
-template <typename T>
-__global__ void __launch_bounds__(256)
-    k_gram_lower(int n, const T* __restrict__ X, T* __restrict__ Ainv) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)n * n) return;
-  const int i = (int)(t / n), j = (int)(t % n);
-  T s = T(0);
-  for (int m = max(i, j); m < n; ++m) s += X[(size_t)m * n + i] * X[(size_t)m * n + j];
-  Ainv[t] = s;
-}
-
 // y = A x with the matrix (and the accumulation) in TA and the vectors in TV
 template <typename TA, typename TV>
 __global__ void __launch_bounds__(256)
@@ -782,62 +548,6 @@ cudaError_t launch_dense_assemble(int dim, int t, int ta, const GridP& g, const 
     return dim == 2 ? dense_t<2, float, float>(g, mask, Kc, A, shift, s)
                     : dense_t<3, float, float>(g, mask, Kc, A, shift, s);
   return cudaErrorInvalidValue;
-}
-
-// The blocked kernels' dynamic shared memory limit is set once, to the most
-// the device allows next to the kernel's static shared memory, not to each
-// call's own size: contexts of different sizes run their set-up from
-// different host threads, and a limit lowered by one thread between another
-// thread's setting and launch would reject that launch.
-template <typename K>
-static int raise_dyn_smem_limit(K kernel) {
-  int dev = 0, optin = 0;
-  cudaFuncAttributes fa;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-      cudaFuncGetAttributes(&fa, kernel) != cudaSuccess)
-    return 48 * 1024;
-  const int lim = optin - (int)fa.sharedSizeBytes;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) ==
-                 cudaSuccess
-             ? lim
-             : 48 * 1024;
-}
-
-template <typename T>
-static cudaError_t cholinv_t(int n, void* A, void* Ainv, int* status, cudaStream_t s) {
-  const size_t smem = (size_t)(CB * CBP + (size_t)n * CBP) * sizeof(T);
-  static const int chol_lim = raise_dyn_smem_limit(k_cholesky_blocked<T>);
-  static const int inv_lim = raise_dyn_smem_limit(k_lower_inverse_blocked<T>);
-  cudaError_t e;
-  if (smem <= (size_t)chol_lim) {
-    k_cholesky_blocked<T><<<1, 1024, smem, s>>>(n, (T*)A, status);
-  } else {
-    k_cholesky<T><<<1, 1024, 0, s>>>(n, (T*)A, status);
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // Ainv is used as scratch for L^{-1} first, then A receives X^T X and
-  // the buffers are swapped by copying back.
-  const int nbk = (n + 31) / 32;
-  const size_t ismem = ((size_t)nbk * 32 * 32 + 32 * 33) * sizeof(T);
-  if (ismem <= (size_t)inv_lim) {
-    k_lower_inverse_blocked<T><<<nbk, 1024, ismem, s>>>(n, (const T*)A, (T*)Ainv);
-  } else {
-    k_lower_inverse<T><<<nblocks((long long)n * 32, 256), 256, 0, s>>>(n, (const T*)A, (T*)Ainv);
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_gram_lower<T><<<nblocks((long long)n * n, 256), 256, 0, s>>>(n, (const T*)Ainv, (T*)A);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyAsync(Ainv, A, sizeof(T) * (size_t)n * n, cudaMemcpyDeviceToDevice, s);
-}
-
-cudaError_t launch_cholesky_inverse(int t, int n, void* A, void* Ainv, int* status,
-                                    cudaStream_t s) {
-  return t == T_F64 ? cholinv_t<double>(n, A, Ainv, status, s)
-                    : cholinv_t<float>(n, A, Ainv, status, s);
 }
 
 cudaError_t launch_dense_gemv(int ta, int t, int n, const void* A, const void* x, void* y,

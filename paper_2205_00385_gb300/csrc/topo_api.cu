@@ -351,6 +351,7 @@ static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
   // the float64 path, and of the mixed path's coarse factorisation)
   void* Ad = cv.take<char>((size_t)nc * nc * 8);
   void* Ai = cv.take<char>((size_t)nc * nc * 8);
+  void* Aw = cv.take<char>((size_t)coarse_scratch_values(nc) * 8);
   if (c) {
     c->E64 = E64; c->Eprev64 = Ep64; c->dE64 = dE64; c->rho_phys = rho; c->invHs = invHs; c->oc_a = oca;
     c->oc_lo = oclo; c->oc_hi = ochi; c->oc_a2 = oca2; c->oc_dv2 = ocdv2;
@@ -363,7 +364,7 @@ static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
     c->partials = partials; c->counters = counters; c->scal = scal; c->small = small;
     c->ints = ints;
     for (int l = 0; l < L; ++l) c->lv[l] = lv[l];
-    c->Adense = Ad; c->Ainv = Ai;
+    c->Adense = Ad; c->Ainv = Ai; c->Awork = Aw;
     c->nc = (int)nc;
   }
   return cv.off;
@@ -796,7 +797,8 @@ static to_status build_hierarchy(to_ctx* c) {
     // regions at Emin / E0 = 1e-9) the float32 coarsest matrix can lose
     // positive definiteness; the context then factors it in float64 from
     // here on (the V-cycles captured with the float32 product are dropped)
-    LAUNCH(c, launch_cholesky_inverse(T_F32, c->nc, c->Adense, c->Ainv, c->ints + I_COARSE, s),
+    LAUNCH(c, launch_cholesky_inverse(T_F32, c->nc, c->Adense, c->Ainv, c->Awork,
+                                      c->ints + I_COARSE, s),
            "coarse factor");
     int bad = 0;
     CUDA_TRY(c, cudaMemcpyAsync(&bad, c->ints + I_COARSE, sizeof(int), cudaMemcpyDeviceToHost, s),
@@ -813,8 +815,8 @@ static to_status build_hierarchy(to_ctx* c) {
     }
   }
   if (c->coarse_t != T_F32)
-    LAUNCH(c, launch_cholesky_inverse(c->coarse_t, c->nc, c->Adense, c->Ainv, c->ints + I_STATUS,
-                                      s), "coarse factor");
+    LAUNCH(c, launch_cholesky_inverse(c->coarse_t, c->nc, c->Adense, c->Ainv, c->Awork,
+                                      c->ints + I_STATUS, s), "coarse factor");
   c->hier_stale = false;
   return TO_OK;
 }

@@ -326,6 +326,7 @@ struct to_ctx {
   // coarsest level
   void* Adense;
   void* Ainv;
+  void* Awork;           // scratch of its inversion
   // reductions and scalars
   double* partials;
   unsigned* counters;
