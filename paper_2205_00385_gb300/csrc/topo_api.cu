@@ -293,6 +293,23 @@ struct Carver {
   }
 };
 
+// Whether level 1 of a 3D hierarchy of >= 3 grids keeps its assembled
+// stencil.  Its implicit form (k_apply3_col, OPK_GAL1) reads only the eight
+// child moduli of a coarse element but spends ~2000 FMAs on it, the stencil
+// 243 FMAs and 84 x 3 values per node.  In float64 (one FMA per clock per SM)
+// the FP64 pipe bounds the implicit form at every size: a V-cycle takes 466 us
+// with it and 171 us with the stencil at 48 x 24 x 24, 2267 and 1291 us at
+// 128 x 64 x 64.  It stays only beyond 8 GB, where the stencil and the element
+// matrices it is assembled from would crowd out the rest of the workspace.
+// In float32 level 1 is always implicit: the stencil gains 10 us of 90 at
+// 96 x 48 x 48 and loses from 128 x 64 x 64 on, and its rounded rows no longer
+// annihilate rigid motions, which costs iterations on designs with solid
+// parts hanging in near-void.
+static bool store_level1(const to_mesh_desc& d) {
+  return d.precision == TO_FP64 &&
+         8.0 * (double)stencil_values(3, T_F64, level_grid(d, 1)) <= 8e9;
+}
+
 static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
   Carver cv{base};
   const int dim = d.dim, npe = 1 << dim, nd = dim * npe, L = d.mg_levels;
@@ -318,11 +335,12 @@ static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
   float* tc_bmat = dim == 3 ? cv.take<float>(2048) : nullptr;
   double* Qc64 = cv.take<double>((size_t)npe * nd * nd);
   float* Qc32 = cv.take<float>((size_t)npe * nd * nd);
-  // 3D with >= 3 levels: level 1 is applied without stored matrices and
-  // level 2 is formed from 64 grandchild tables
-  const bool l1_implicit = dim == 3 && L >= 3;
-  double* R2_64 = l1_implicit ? cv.take<double>((size_t)64 * 576) : nullptr;
-  float* R2_32 = l1_implicit ? cv.take<float>((size_t)64 * 576) : nullptr;
+  // 3D with >= 3 levels: level 2 is formed from 64 grandchild tables, and
+  // level 1 may be applied without stored matrices
+  const bool l2_tables = dim == 3 && L >= 3;
+  const bool l1_implicit = l2_tables && !store_level1(d);
+  double* R2_64 = l2_tables ? cv.take<double>((size_t)64 * 576) : nullptr;
+  float* R2_32 = l2_tables ? cv.take<float>((size_t)64 * 576) : nullptr;
   double* partials = cv.take<double>((size_t)RED_BLOCKS * MAXB * MAXB);
   unsigned* counters = cv.take<unsigned>(C_NCOUNTERS);
   double* scal = cv.take<double>(S_NSLOTS);
@@ -360,7 +378,7 @@ static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
     c->Phi = Phi; c->KPhi = KPhi; c->R = R; c->Q = Q; c->t = t;
     c->Qc64 = Qc64; c->Qc32 = Qc32;
     c->tc_bmat = tc_bmat;
-    c->l1_implicit = l1_implicit; c->R2_64 = R2_64; c->R2_32 = R2_32;
+    c->l2_tables = l2_tables; c->l1_implicit = l1_implicit; c->R2_64 = R2_64; c->R2_32 = R2_32;
     c->partials = partials; c->counters = counters; c->scal = scal; c->small = small;
     c->ints = ints;
     for (int l = 0; l < L; ++l) c->lv[l] = lv[l];
@@ -525,7 +543,7 @@ to_status to_mesh_init(const to_mesh_desc* desc, const uint8_t* fixed_mask, cons
     INIT_TRY(cudaStreamSynchronize(s), "sync");
     INIT_TRY(tc_prepare(), "tensor-core operator set-up");
   }
-  if (c->l1_implicit) {
+  if (c->l2_tables) {
     std::vector<double> R2((size_t)64 * 576);
     grandchild_galerkin(Qc.data(), R2.data());
     std::vector<float> R2f(R2.size());
@@ -691,6 +709,8 @@ static ApplyArgs fine_args(const to_ctx* c, int op, int tc, int tx, int ty, cons
   return a;
 }
 
+static void implicit_level1(const to_ctx* c, ApplyArgs* a);
+
 static ApplyArgs coarse_args(const to_ctx* c, int l, const void* x, void* y, const void* b,
                              int epi) {
   ApplyArgs a;
@@ -710,16 +730,6 @@ static ApplyArgs coarse_args(const to_ctx* c, int l, const void* x, void* y, con
   a.gf = c->lv[0].g;
   a.S = c->lv[l].S;
   a.colfix = c->lv[l].colfix;
-  if (l == 1 && c->l1_implicit) {
-    // level-1 Galerkin operator evaluated from the finest moduli
-    a.expl = false;
-    a.gal1 = true;
-    a.coef = t == T_F64 ? (const void*)c->E64 : (const void*)c->E32;
-    a.Kc = nullptr;
-    a.wht = t == T_F64 ? (const void*)c->wht64 : (const void*)c->wht32;
-    a.zsplit = epi == EPI_RESID ? c->tuned_zc[TO_TUNE_GAL1_RESID]
-             : epi == EPI_SMOOTH ? c->tuned_zc[TO_TUNE_GAL1_SMOOTH] : 0;
-  }
   a.x = x;
   a.y = y;
   a.b = b;
@@ -727,7 +737,20 @@ static ApplyArgs coarse_args(const to_ctx* c, int l, const void* x, void* y, con
   a.omega = 0.6;
   a.dfix = 1.0;
   a.epi = epi;
+  if (l == 1 && c->l1_implicit) implicit_level1(c, &a);
   return a;
+}
+
+// makes the arguments of a level-1 product those of the Galerkin operator
+// evaluated from the finest moduli
+static void implicit_level1(const to_ctx* c, ApplyArgs* a) {
+  a->expl = false;
+  a->gal1 = true;
+  a->coef = a->tc == T_F64 ? (const void*)c->E64 : (const void*)c->E32;
+  a->Kc = nullptr;
+  a->wht = a->tc == T_F64 ? (const void*)c->wht64 : (const void*)c->wht32;
+  a->zsplit = a->epi == EPI_RESID ? c->tuned_zc[TO_TUNE_GAL1_RESID]
+            : a->epi == EPI_SMOOTH ? c->tuned_zc[TO_TUNE_GAL1_SMOOTH] : 0;
 }
 
 // Algorithmic DRAM bytes of one operator launch: every input and output
@@ -768,18 +791,20 @@ static to_status build_hierarchy(to_ctx* c) {
   LAUNCH(c, launch_diag(c->dim, c->lv[0].g, c->lv[0].mask, t, false, E, nullptr, KE,
                         c->lv[0].dinv, s, c->springs), "diag 0");
   if (c->l1_implicit) {
-    // level 1 stays implicit; level 2 straight from the finest moduli
-    const void* R2 = t == T_F64 ? (const void*)c->R2_64 : (const void*)c->R2_32;
     LAUNCH(c, launch_diag_l1(t, c->lv[1].g, c->lv[0].g, c->lv[1].mask, c->qdiag, E,
                              c->lv[1].dinv, s), "diag 1");
-    LAUNCH(c, launch_galerkin_l2(t, c->lv[2].g, c->lv[0].g, E, R2, c->lv[2].Kc, s), "galerkin 2");
   } else {
     LAUNCH(c, launch_galerkin_fine(c->dim, t, c->lv[1].g, c->lv[0].g, E, Qc, c->lv[1].Kc, s),
            "galerkin 1");
     LAUNCH(c, launch_spring_galerkin(c->dim, t, c->lv[1].g, c->lv[0].g, c->springs, c->lv[1].Kc,
                                      s), "springs 1");
   }
-  const int lfirst = c->l1_implicit ? 3 : 2;
+  if (c->l2_tables) {
+    // level 2 straight from the finest moduli
+    const void* R2 = t == T_F64 ? (const void*)c->R2_64 : (const void*)c->R2_32;
+    LAUNCH(c, launch_galerkin_l2(t, c->lv[2].g, c->lv[0].g, E, R2, c->lv[2].Kc, s), "galerkin 2");
+  }
+  const int lfirst = c->l2_tables ? 3 : 2;
   for (int l = lfirst; l < c->L; ++l)
     LAUNCH(c, launch_galerkin_coarse(c->dim, t, c->lv[l].g, c->lv[l - 1].g, c->lv[l - 1].Kc,
                                      c->lv[l].Kc, s), "galerkin l");
@@ -1481,9 +1506,10 @@ to_status to_autotune(to_ctx* c, int32_t reps, to_tune_result* results, int32_t 
         return true;
       case TO_TUNE_GAL1_RESID:
       case TO_TUNE_GAL1_SMOOTH:
-        if (!c->l1_implicit) return false;
+        if (!c->l2_tables) return false;
         *a = coarse_args(c, 1, lv[1].z, kind == TO_TUNE_GAL1_RESID ? lv[1].r : lv[1].z2, lv[1].b,
                          kind == TO_TUNE_GAL1_RESID ? EPI_RESID : EPI_SMOOTH);
+        implicit_level1(c, a);   // (also where this context stores level 1)
         a->clean_inputs = true;
         return true;
       case TO_TUNE_ACC_APPLY:

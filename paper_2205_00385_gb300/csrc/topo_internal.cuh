@@ -316,9 +316,9 @@ struct to_ctx {
   // Galerkin tables (level-1 child matrices Q_c), float64 and float32
   double* Qc64;
   float* Qc32;
-  // 3D, >= 3 levels: level 1 applied from the finest moduli (no stored
-  // matrices); level 2 formed with the 64 grandchild tables R2
-  bool l1_implicit;
+  // 3D, >= 3 levels: level 2 formed with the 64 grandchild tables R2, and,
+  // unless its stencil is stored, level 1 applied from the finest moduli
+  bool l2_tables, l1_implicit;
   bool df_ok;          // double-float finest-grid operator available (3D)
   double* R2_64;
   float* R2_32;
