@@ -293,25 +293,18 @@ cudaError_t launch_oc_prep(long long nel, const double* rho, const double* dc,
 cudaError_t launch_oc_step(long long nel, const double* rho, const double* a,
                            const double* dv, double move, double target, double* scal,
                            double* partials, unsigned* counter, cudaStream_t s);
-// bisection with stored move-limit bounds lo/hi (context path)
-cudaError_t launch_oc_prep_b(long long nel, const double* rho, const double* dc,
-                             const double* dv, double move, double* a, double* lo, double* hi,
-                             double* scal, cudaStream_t s);
-cudaError_t launch_oc_step_b(long long nel, const double* a, const double* lo, const double* hi,
-                             const double* dv, double target, double* scal, double* partials,
-                             unsigned* counter, cudaStream_t s);
 // lambda search of the OC update: the candidate factors
 // a = rho max(0, -dc/dv)^eta (float64 copy a64 for the final update; eta
-// 1/2 for compliance) and the move limits and dv as double-float pairs; one
-// launch narrows [l1, l2] eight-fold in double-float; rho_new =
-// clamp(a lambda^-eta)
+// 1/2 for compliance), the move limits and dv as double-float pairs and the
+// first bracket; one sweep narrows the bracket in double-float (a no-op once
+// it is within 1e-13); rho_new = clamp(a lambda^-eta)
 cudaError_t launch_oc_prep_d(long long nel, const double* rho, const double* dc,
-                             const double* dv, double move, double* a64, void* a2, void* lo2,
-                             void* hi2, void* dv2, double* scal, cudaStream_t s,
-                             double eta = 0.5);
-cudaError_t launch_oc_section(long long nel, const void* a2, const void* lo2, const void* hi2,
-                              const void* dv2, double target, double* scal, double* partials,
-                              unsigned* counter, cudaStream_t s, double eta = 0.5);
+                             const double* dv, double move, double target, double* a64, void* a2,
+                             void* lo2, void* hi2, void* dv2, double* scal, double* partials,
+                             unsigned* counter, cudaStream_t s, double eta = 0.5);
+cudaError_t launch_oc_sweep(long long nel, const void* a2, const void* lo2, const void* hi2,
+                            const void* dv2, double target, double* scal, double* partials,
+                            unsigned* counter, cudaStream_t s, double eta = 0.5);
 cudaError_t launch_oc_final(long long nel, double* rho, const double* a, double move,
                             double* scal, double* change_dev, double* partials,
                             unsigned* counter, cudaStream_t s, double eta = 0.5);

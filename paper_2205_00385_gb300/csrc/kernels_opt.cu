@@ -4,6 +4,8 @@
 // multiplier.  All float64.
 #include <math.h>
 
+#include <algorithm>
+
 #include "dfmath.cuh"
 #include "kernels.h"
 
@@ -300,59 +302,25 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
 }
 
-// Context path: the move-limit bounds are stored once, so a bisection step
-// costs one multiply, two clamps and one multiply-add in float64 per element
-// (same values as k_oc_step, which recomputes them).
-__global__ void __launch_bounds__(256)
-    k_oc_prep_b(long long nel, const double* __restrict__ rho, const double* __restrict__ dc,
-                const double* __restrict__ dv, double move, double* __restrict__ a,
-                double* __restrict__ lo, double* __restrict__ hi, double* scal) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e == 0) {
-    scal[S_OC_L1] = 0.0;
-    scal[S_OC_L2] = 1e9;
-  }
-  if (e >= nel) return;
-  const double r = rho[e];
-  a[e] = r * sqrt(fmax(0.0, -dc[e] / dv[e]));
-  lo[e] = fmax(0.0, r - move);
-  hi[e] = fmin(1.0, r + move);
-}
-
-__global__ void __launch_bounds__(RED_THREADS)
-    k_oc_step_b(long long nel, const double* __restrict__ a, const double* __restrict__ lo,
-                const double* __restrict__ hi, const double* __restrict__ dv, double target,
-                double* scal, double* partials, unsigned* counter) {
-  __shared__ double sh[32];
-  const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
-  if (!((l2 - l1) > 1e-13 * (l1 + l2))) return;
-  const double lmid = 0.5 * (l1 + l2);
-  const double s = 1.0 / sqrt(lmid);
-  double v[1] = {0.0};
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nel;
-       e += (long long)gridDim.x * blockDim.x)
-    v[0] = fma(dv[e], fmin(hi[e], fmax(lo[e], a[e] * s)), v[0]);
-  block_sum<1>(v, sh);
-  if (publish_partials<1>(v, partials, counter)) {
-    double o[1];
-    finish_sum<1>(partials, counter, o, sh);
-    if (threadIdx.x == 0) {
-      if (o[0] > target)
-        scal[S_OC_L1] = lmid;
-      else
-        scal[S_OC_L2] = lmid;
-      scal[S_OC_VOL] = o[0];
-    }
-  }
-}
-
-// Context path of the mixed and float64 solvers alike: the lambda search
-// runs as an OC_SPLIT-way section per pass in double-float on the FP32 pipe
-// (the volume at OC_SPLIT - 1 interior points of [l1, l2] is summed for
-// every element in one sweep, and the sub-interval holding the root is
-// kept), 3 bits of bracket per sweep against 1 for a float64 bisection
-// step.  It stops at the same relative bracket of 1e-13.
-constexpr int OC_SPLIT = 8;
+// Context path of the mixed and float64 solvers alike: the search for the
+// multiplier lambda.  The volume is a non-decreasing, piecewise linear
+// function of s = lambda^-eta, so after a bracket [l1, l2] with
+// V(l1) > target >= V(l2) is narrow, the secant point of the bracket is off by
+// about the square of its width.  A sweep sums the volume at OC_NP points of
+// the bracket in double-float; its last block keeps the sub-interval that
+// holds the root and writes the next points:
+//   first sweep      around the multiplier that no limit would clamp, l0 8^j
+//   lower end 0      l2 / 8^7 .. l2 / 8
+//   ratio above 4    geometric
+//   narrow           the secant point, +- guards of half the squared width and
+//                    1/32 of that, and the bracket's thirds, which bound the
+//                    sweeps when the secant point misses
+// Six or seven sweeps reach the relative bracket of 1e-13 (equal sections of
+// the bracket took 17 to 23); a sweep after that is a no-op.  A sweep reads
+// 32 bytes per element (57 MB at 192 x 96 x 96, which stays in L2).
+constexpr int OC_NP = 7, OC_T = 512, OC_BLOCKS = 304;
+constexpr double OC_LAM_MAX = 1e9;
+static_assert(OC_NP <= S_OC_NPT && OC_NP <= OC_T / 32, "one warp per point");
 
 // x^eta of the OC rule (sqrt for the compliance rule's eta = 1/2) and the
 // multiplier's factor lambda^-eta
@@ -362,92 +330,199 @@ __device__ __forceinline__ double oc_damp(double x, double eta) {
 __device__ __forceinline__ double oc_lam_factor(double lam, double eta) {
   return eta == 0.5 ? 1.0 / sqrt(lam) : pow(lam, -eta);
 }
-
-__global__ void __launch_bounds__(256)
-    k_oc_prep_d(long long nel, const double* __restrict__ rho, const double* __restrict__ dc,
-                const double* __restrict__ dv, double move, double* __restrict__ a64,
-                float2* __restrict__ a, float2* __restrict__ lo, float2* __restrict__ hi,
-                float2* __restrict__ dvd, double* scal, double eta) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e == 0) {
-    scal[S_OC_L1] = 0.0;
-    scal[S_OC_L2] = 1e9;
-  }
-  if (e >= nel) return;
-  const double r = rho[e];
-  const double ae = r * oc_damp(fmax(0.0, -dc[e] / dv[e]), eta);
-  a64[e] = ae;
-  const dfl av = split_d(ae);
-  const dfl lv = split_d(fmax(0.0, r - move)), hv = split_d(fmin(1.0, r + move));
-  const dfl dd = split_d(dv[e]);
-  a[e] = make_float2(av.h, av.l);
-  lo[e] = make_float2(lv.h, lv.l);
-  hi[e] = make_float2(hv.h, hv.l);
-  dvd[e] = make_float2(dd.h, dd.l);
+__device__ __forceinline__ double oc_lam_of(double s, double eta) {
+  return eta == 0.5 ? 1.0 / (s * s) : pow(s, -1.0 / eta);
 }
 
-// Section point j (1 .. OC_SPLIT-1) of the bracket [l1, l2]: evenly spaced,
-// or, while the lower end is still 0, geometric (l2 / 8^(OC_SPLIT - j)), which
-// brings an upper end far above lambda down by up to 8^7 per sweep; point
-// OC_SPLIT is l2 itself.
-__device__ __forceinline__ double oc_point(double l1, double l2, int j) {
-  if (j >= OC_SPLIT) return l2;
-  if (l1 == 0.0) return ldexp(l2, -3 * (OC_SPLIT - j));
-  return l1 + (double)j * ((l2 - l1) / OC_SPLIT);
-}
-
-__global__ void __launch_bounds__(RED_THREADS)
-    k_oc_section(long long nel, const float2* __restrict__ a, const float2* __restrict__ lo,
-                 const float2* __restrict__ hi, const float2* __restrict__ dvd, double target,
-                 double* scal, double* partials, unsigned* counter, double eta) {
-  constexpr int NP = OC_SPLIT - 1;
-  __shared__ double sh[NP * 32];
-  __shared__ dfl s_s[NP];
-  const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
-  if (!((l2 - l1) > 1e-13 * (l1 + l2))) return;
-  if (threadIdx.x < NP) {
-    const double lam = oc_point(l1, l2, threadIdx.x + 1);
-    s_s[threadIdx.x] = split_d(oc_lam_factor(lam, eta));
+// Sums of NV double-float values per thread over the grid, finished by the
+// last block: warps reduce in double-float, then one warp per value adds the
+// warp results, and in the last block the block results, in float64 in a
+// fixed order.  Returns true in the last block, where out[] (shared) is set.
+template <int NV>
+__device__ __forceinline__ bool oc_grid_sum(const dfl (&v)[NV], double (&out)[NV],
+                                            double (&sh)[NV][OC_T / 32], double* partials,
+                                            unsigned* counter) {
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    dfl x = v[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const dfl y = {__shfl_down_sync(0xffffffffu, x.h, o), __shfl_down_sync(0xffffffffu, x.l, o)};
+      x = df_add(x, y);
+    }
+    if (lane == 0) sh[q][warp] = df_to_d(x);
   }
   __syncthreads();
-  dfl sv[NP], v[NP];
+  if (warp < NV) {
+    double t = lane < OC_T / 32 ? sh[warp][lane] : 0.0;
 #pragma unroll
-  for (int j = 0; j < NP; ++j) {
-    sv[j] = s_s[j];
+    for (int o = OC_T / 64; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) partials[(size_t)blockIdx.x * NV + warp] = t;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  if (warp < NV) {
+    double t = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += partials[(size_t)b * NV + warp];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) out[warp] = t;
+  }
+  if (threadIdx.x == 0) *counter = 0u;
+  __syncthreads();
+  return true;
+}
+
+// bracket within its final width (also when both ends are 0)
+__device__ __forceinline__ bool oc_done(double l1, double l2) {
+  return !((l2 - l1) > 1e-13 * (l1 + l2));
+}
+
+// Writes the bracket and its next points; called by one whole warp.
+__device__ __forceinline__ void oc_next_points(double l1, double l2, double v1, double v2,
+                                               double target, double eta, double l0,
+                                               double* scal) {
+  const int j = threadIdx.x & 31;
+  double lam;
+  if (l0 > 0.0) {
+    lam = fmin(ldexp(l0, 3 * (j - OC_NP / 2)), l2);
+  } else if (l1 == 0.0) {
+    lam = ldexp(l2, -3 * (OC_NP - j));
+  } else if (l2 > 4.0 * l1) {
+    const double q = sqrt(sqrt(sqrt(l2 / l1)));
+    lam = l1;
+    for (int i = 0; i <= j && i < OC_NP; ++i) lam *= q;
+  } else if (!(v1 > v2)) {   // a volume not known (or no slope): equal sections
+    lam = l1 + (j + 1) * ((l2 - l1) / (OC_NP + 1));
+  } else {
+    const double sa = oc_lam_factor(l2, eta), sb = oc_lam_factor(l1, eta);
+    const double mid = oc_lam_of(sa + (target - v2) * ((sb - sa) / (v1 - v2)), eta);
+    const double w = (l2 - l1) / l2, d = mid * fmax(0.5 * w * w, 6.4e-13);
+    lam = j == 0 ? mid - d
+        : j == 1 ? mid - d / 32
+        : j == 2 ? mid
+        : j == 3 ? mid + d / 32
+        : j == 4 ? mid + d
+                 : l1 + (j - 4) * ((l2 - l1) / 3);
+  }
+  lam = fmin(fmax(lam, l1), l2);
+  // ascending order: the rank of each point among the OC_NP
+  int rank = 0;
+#pragma unroll
+  for (int i = 0; i < OC_NP; ++i) {
+    const double o = __shfl_sync(0xffffffffu, lam, i);
+    rank += o < lam || (o == lam && i < j);
+  }
+  if (j < OC_NP) {
+    scal[S_OC_PT + rank] = lam;
+    scal[S_OC_SP + rank] = oc_lam_factor(lam, eta);
+  }
+  if (j == 0) {
+    scal[S_OC_L1] = l1;
+    scal[S_OC_L2] = l2;
+    scal[S_OC_V1] = v1;
+    scal[S_OC_V2] = v2;
+  }
+}
+
+// a_e = rho_e max(0, -dc_e / dv_e)^eta, the move limits and the weights as
+// pairs, the search's bracket [0, 1e9] and its first points.  When even the
+// upper limits hold no more than the target volume the bracket is 0, and
+// when its upper end still holds more, that end.
+__global__ void __launch_bounds__(OC_T)
+    k_oc_prep_d(long long nel, const double* __restrict__ rho, const double* __restrict__ dc,
+                const double* __restrict__ dv, double move, double target,
+                double* __restrict__ a64, float2* __restrict__ a, float2* __restrict__ lo,
+                float2* __restrict__ hi, float2* __restrict__ dvd, double* scal, double eta,
+                double* partials, unsigned* counter) {
+  __shared__ double sh[3][OC_T / 32], tot[3];
+  __shared__ dfl s_top;
+  if (threadIdx.x == 0) s_top = split_d(oc_lam_factor(OC_LAM_MAX, eta));
+  __syncthreads();
+  const dfl top = s_top;
+  dfl v[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  for (long long e = (long long)blockIdx.x * OC_T + threadIdx.x; e < nel;
+       e += (long long)gridDim.x * OC_T) {
+    const double r = rho[e], d = dv[e];
+    const double ae = r * oc_damp(fmax(0.0, -dc[e] / d), eta);
+    a64[e] = ae;
+    const dfl av = split_d(ae);
+    const dfl lv = split_d(fmax(0.0, r - move)), hv = split_d(fmin(1.0, r + move));
+    const dfl dd = split_d(d);
+    a[e] = make_float2(av.h, av.l);
+    lo[e] = make_float2(lv.h, lv.l);
+    hi[e] = make_float2(hv.h, hv.l);
+    dvd[e] = make_float2(dd.h, dd.l);
+    df_dot_acc(v[0], dd, av);
+    df_dot_acc(v[1], dd, av.h > 0.f ? hv : lv);
+    const dfl x = df_mul(av, top);
+    df_dot_acc(v[2], dd, df_gt(x, hv) ? hv : (df_gt(lv, x) ? lv : x));
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) v[q] = df_norm(v[q]);
+  if (!oc_grid_sum<3>(v, tot, sh, partials, counter) || threadIdx.x >= 32) return;
+  const double l0 = oc_lam_of(target / tot[0], eta);
+  const double l1 = tot[1] > target && tot[2] > target ? OC_LAM_MAX : 0.0;
+  const double l2 = tot[1] > target ? OC_LAM_MAX : 0.0;
+  oc_next_points(l1, l2, tot[1], tot[2], target, eta,
+                 l0 > 1e-60 && l0 < OC_LAM_MAX ? l0 : 0.0, scal);
+}
+
+__global__ void __launch_bounds__(OC_T, 2)
+    k_oc_sweep(long long nel, const float4* __restrict__ a, const float4* __restrict__ lo,
+               const float4* __restrict__ hi, const float4* __restrict__ dvd, double target,
+               double* scal, double* partials, unsigned* counter, double eta) {
+  __shared__ double sh[OC_NP][OC_T / 32], tot[OC_NP];
+  pdl_wait();
+  const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
+  if (oc_done(l1, l2)) return;
+  dfl sv[OC_NP], v[OC_NP];
+#pragma unroll
+  for (int j = 0; j < OC_NP; ++j) {
+    sv[j] = split_d(scal[S_OC_SP + j]);
     v[j] = {0.f, 0.f};
   }
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nel;
-       e += (long long)gridDim.x * blockDim.x) {
-    const float2 a2 = a[e], l2v = lo[e], h2 = hi[e], d2 = dvd[e];
-    const dfl av = {a2.x, a2.y}, lv = {l2v.x, l2v.y}, hv = {h2.x, h2.y}, dd = {d2.x, d2.y};
+  auto element = [&](dfl av, dfl lv, dfl hv, dfl dd) {
 #pragma unroll
-    for (int j = 0; j < NP; ++j) {
+    for (int j = 0; j < OC_NP; ++j) {
       dfl x = df_mul(av, sv[j]);
       x = df_gt(x, hv) ? hv : (df_gt(lv, x) ? lv : x);
       df_dot_acc(v[j], dd, x);
     }
+  };
+  // two elements per 16-byte load (nel is even: every grid coarsens once)
+  for (long long q = (long long)blockIdx.x * OC_T + threadIdx.x; 2 * q < nel;
+       q += (long long)gridDim.x * OC_T) {
+    const float4 a4 = a[q], l4 = lo[q], h4 = hi[q], d4 = dvd[q];
+    element({a4.x, a4.y}, {l4.x, l4.y}, {h4.x, h4.y}, {d4.x, d4.y});
+    element({a4.z, a4.w}, {l4.z, l4.w}, {h4.z, h4.w}, {d4.z, d4.w});
   }
 #pragma unroll
-  for (int j = 0; j < NP; ++j) v[j] = df_norm(v[j]);
-  double o1[NP];
-  block_sum_df<NP>(v, o1, sh);
-  if (publish_partials<NP>(o1, partials, counter)) {
-    double o[NP];
-    finish_sum<NP>(partials, counter, o, sh);
-    if (threadIdx.x == 0) {
-      // the volume decreases with lambda: keep the last point above target
-      // and the first at or below it
-      int k = 0;
-      while (k < NP && o[k] > target) ++k;
-      const double nl1 = k > 0 ? oc_point(l1, l2, k) : l1;
-      const double nl2 = oc_point(l1, l2, k + 1);
-      scal[S_OC_L1] = nl1;
-      scal[S_OC_L2] = nl2;
-      scal[S_OC_VOL] = k > 0 ? o[k - 1] : o[0];
-    }
-  }
+  for (int j = 0; j < OC_NP; ++j) v[j] = df_norm(v[j]);
+  pdl_launch_dependents();
+  if (!oc_grid_sum<OC_NP>(v, tot, sh, partials, counter) || threadIdx.x >= 32) return;
+  // the volume decreases with lambda: keep the last point above target and
+  // the first at or below it
+  int k = 0;
+  while (k < OC_NP && tot[k] > target) ++k;
+  const double n1 = k > 0 ? scal[S_OC_PT + k - 1] : l1;
+  const double w1 = k > 0 ? tot[k - 1] : scal[S_OC_V1];
+  const double n2 = k < OC_NP ? scal[S_OC_PT + k] : l2;
+  const double w2 = k < OC_NP ? tot[k] : scal[S_OC_V2];
+  __syncwarp();
+  oc_next_points(n1, n2, w1, w2, target, eta, 0.0, scal);
 }
 
+// rho <- clamp(a lambda^-eta) and max |rho_new - rho|.  The limits are
+// selected by comparing bit patterns as integers (doubles of one sign order as
+// their bits do), which leaves four FP64 instructions per element; a product
+// that is not a number (0 x infinity) takes the lower limit, as fmax does.
 __global__ void __launch_bounds__(RED_THREADS)
     k_oc_final(long long nel, double* __restrict__ rho, const double* __restrict__ a,
                double move, double* scal, double* change_dev, double* partials,
@@ -455,14 +530,23 @@ __global__ void __launch_bounds__(RED_THREADS)
   __shared__ double sh[32];
   const double lam = 0.5 * (scal[S_OC_L1] + scal[S_OC_L2]);
   const double s = oc_lam_factor(lam, eta);
-  double v[1] = {0.0};
+  const long long inf = 0x7ff0000000000000LL, one = __double_as_longlong(1.0);
+  long long most = 0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nel;
        e += (long long)gridDim.x * blockDim.x) {
     const double r = rho[e];
-    const double rn = oc_new(a[e], s, r, move);
+    long long lo = __double_as_longlong(r - move), hi = __double_as_longlong(r + move);
+    long long t = __double_as_longlong(a[e] * s);
+    lo = lo < 0 || lo > inf ? 0 : lo;
+    hi = hi > one ? one : hi;
+    t = t < lo || t > inf ? lo : t;
+    t = t > hi ? hi : t;
+    const double rn = __longlong_as_double(t);
     rho[e] = rn;
-    v[0] = fmax(v[0], fabs(rn - r));
+    const long long d = __double_as_longlong(rn - r) & 0x7fffffffffffffffLL;
+    if (d <= inf && d > most) most = d;
   }
+  double v[1] = {__longlong_as_double(most)};
   block_max<1>(v, sh);
   if (publish_partials<1>(v, partials, counter)) {
     double o[1];
@@ -571,37 +655,26 @@ cudaError_t launch_oc_step(long long nel, const double* rho, const double* a,
   return cudaGetLastError();
 }
 
-cudaError_t launch_oc_prep_b(long long nel, const double* rho, const double* dc,
-                             const double* dv, double move, double* a, double* lo, double* hi,
-                             double* scal, cudaStream_t s) {
-  k_oc_prep_b<<<nblocks(nel, 256), 256, 0, s>>>(nel, rho, dc, dv, move, a, lo, hi, scal);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_oc_step_b(long long nel, const double* a, const double* lo, const double* hi,
-                             const double* dv, double target, double* scal, double* partials,
-                             unsigned* counter, cudaStream_t s) {
-  k_oc_step_b<<<RED_BLOCKS, RED_THREADS, 0, s>>>(nel, a, lo, hi, dv, target, scal, partials,
-                                                 counter);
-  return cudaGetLastError();
+static int oc_blocks(long long nel) {
+  return (int)std::min<long long>((nel + 2 * OC_T - 1) / (2 * OC_T), OC_BLOCKS);
 }
 
 cudaError_t launch_oc_prep_d(long long nel, const double* rho, const double* dc,
-                             const double* dv, double move, double* a64, void* a2, void* lo2,
-                             void* hi2, void* dv2, double* scal, cudaStream_t s, double eta) {
-  k_oc_prep_d<<<nblocks(nel, 256), 256, 0, s>>>(nel, rho, dc, dv, move, a64, (float2*)a2,
-                                                (float2*)lo2, (float2*)hi2, (float2*)dv2, scal,
-                                                eta);
+                             const double* dv, double move, double target, double* a64, void* a2,
+                             void* lo2, void* hi2, void* dv2, double* scal, double* partials,
+                             unsigned* counter, cudaStream_t s, double eta) {
+  k_oc_prep_d<<<oc_blocks(nel), OC_T, 0, s>>>(nel, rho, dc, dv, move, target, a64, (float2*)a2,
+                                              (float2*)lo2, (float2*)hi2, (float2*)dv2, scal, eta,
+                                              partials, counter);
   return cudaGetLastError();
 }
 
-cudaError_t launch_oc_section(long long nel, const void* a2, const void* lo2, const void* hi2,
-                              const void* dv2, double target, double* scal, double* partials,
-                              unsigned* counter, cudaStream_t s, double eta) {
-  k_oc_section<<<RED_BLOCKS, RED_THREADS, 0, s>>>(nel, (const float2*)a2, (const float2*)lo2,
-                                                  (const float2*)hi2, (const float2*)dv2, target,
-                                                  scal, partials, counter, eta);
-  return cudaGetLastError();
+cudaError_t launch_oc_sweep(long long nel, const void* a2, const void* lo2, const void* hi2,
+                            const void* dv2, double target, double* scal, double* partials,
+                            unsigned* counter, cudaStream_t s, double eta) {
+  return launch_pdl(k_oc_sweep, dim3(oc_blocks(nel)), dim3(OC_T), 0, s, nel, (const float4*)a2,
+                    (const float4*)lo2, (const float4*)hi2, (const float4*)dv2, target, scal,
+                    partials, counter, eta);
 }
 
 cudaError_t launch_oc_final(long long nel, double* rho, const double* a, double move,
