@@ -92,6 +92,11 @@ int vcycle_coarse_cluster(int dim, int t, int ta);
 cudaError_t launch_vcycle_coarse(int dim, int t, int ta, const VFuseArgs& a, cudaStream_t s);
 // Float32 3D finest-grid operator, two element columns per thread with packed
 // f32x2 arithmetic (kernels_pair.cu); pair_apply_ok tells whether it applies.
+// float64 finest-grid hex8 operator with the element arithmetic in 64-bit
+// fixed point (kernels_fx.cu)
+bool fx_apply_ok(const ApplyArgs& a);
+cudaError_t launch_apply_fx(const ApplyArgs& a, cudaStream_t s);
+void fx_prepare();
 bool pair_apply_ok(const ApplyArgs& a);
 cudaError_t launch_apply_pair(const ApplyArgs& a, cudaStream_t s);
 // caches the pair kernel's resident-block counts for the current device

@@ -1,8 +1,7 @@
 // Float64-accurate hex8 stiffness operator in double-float arithmetic.
 //
-// GB300 runs float64 at one FMA per clock per SM, 1/128 of the float32
-// rate, so the float64 Walsh kernel (k_apply3_col<double>) is bound by the
-// FP64 pipe at ~1.3 ms per 5.4M-DOF apply.  Here every value is an unevaluated sum hi + lo of two
+// GB300 runs float64 at 1/128 of the float32 rate, so a float64 transform is
+// bound by the FP64 pipe.  Here every value is an unevaluated sum hi + lo of two
 // floats (48-bit significand) and all arithmetic runs on the FP32 pipe with
 // error-free transformations (TwoSum, FMA-based TwoProduct).  float64 inputs
 // are split into (hi, lo) and results widened back with integer bit

@@ -626,8 +626,10 @@ static cudaError_t run_col_epi(const ApplyArgs& a, cudaStream_t s) {
 template <int OP>
 static cudaError_t run_col_types(const ApplyArgs& a, cudaStream_t s) {
   if (a.tc == T_F64) {
-    if (a.tx != T_F64 || a.ty != T_F64) return cudaErrorInvalidValue;
-    return run_col_epi<double, double, double, OP>(a, s);
+    // (the finest float64 operator runs in fixed point, kernels_fx.cu)
+    if constexpr (OP == OPK_GAL1)
+      if (a.tx == T_F64 && a.ty == T_F64) return run_col_epi<double, double, double, OP>(a, s);
+    return cudaErrorInvalidValue;
   }
   if (a.tx == T_F32 && a.ty == T_F32) return run_col_epi<float, float, float, OP>(a, s);
   if (OP == OPK_FINE) {
@@ -645,6 +647,7 @@ cudaError_t launch_apply(const ApplyArgs& a, cudaStream_t s) {
     if (a.gal1) return run_col_types<OPK_GAL1>(a, s);
     if (a.use_tc && tc_apply_ok(a)) return launch_apply_tc(a, s);
     if (pair_apply_ok(a)) return launch_apply_pair(a, s);
+    if (fx_apply_ok(a)) return launch_apply_fx(a, s);
     if (a.wht != nullptr) return run_col_types<OPK_FINE>(a, s);
   }
   return a.dim == 2 ? run_apply_dim<2>(a, s) : run_apply_dim<3>(a, s);

@@ -573,6 +573,7 @@ to_status to_mesh_init(const to_mesh_desc* desc, const uint8_t* fixed_mask, cons
     pair_prepare();
     col_prepare();
     df_prepare();
+    fx_prepare();
   }
   // first level of the optional fused coarse stretch (TO_OPERATOR_FUSED_COARSE):
   // the first stored level whose stencil is small (a few MB)
