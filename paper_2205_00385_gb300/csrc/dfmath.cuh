@@ -7,6 +7,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "topo_internal.cuh"
+
 namespace topo {
 
 struct dfl {
@@ -122,6 +124,24 @@ __device__ __forceinline__ void block_sum_df(dfl (&v)[NV], double (&out)[NV], do
     }
   }
   __syncthreads();
+}
+
+// grid_sum of NV double-float values per thread; warps reduce in double-float
+template <int NV, int NW>
+__device__ __forceinline__ bool grid_sum_df(const dfl (&v)[NV], double (&sh)[NV][NW],
+                                            double (&out)[NV], double* partials,
+                                            unsigned* counter) {
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    dfl x = v[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const dfl y = {__shfl_down_sync(0xffffffffu, x.h, o), __shfl_down_sync(0xffffffffu, x.l, o)};
+      x = df_add(x, y);
+    }
+    if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = df_to_d(x);
+  }
+  return grid_sum<NV, NW>(sh, out, partials, counter);
 }
 
 // a > b for normalised pairs

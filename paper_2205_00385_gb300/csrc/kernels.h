@@ -238,13 +238,14 @@ cudaError_t launch_gs_accept(long long n, int vt, void* R, int src, const double
 // Y[:, j] = sum_{i < kq} U[i + MAXB j] Q[:, i] for j < k <= kq (Y != Q)
 cudaError_t launch_combine_multi(long long n, int vt, const void* Q, int kq, const double* U,
                                  int k, void* Y, cudaStream_t s);
-// mixed-path CG (pairs x, r, p; float32 shadows p32 -> q32 and z32)
+// mixed-path CG (pairs x, r, p; float32 shadows p32 -> q32 and z32; vectors of
+// the workspace, 16-byte aligned): out = a . b
 cudaError_t launch_dot_d2f(long long n, const void* a, const float* b, double* partials,
                            unsigned* counter, double* out, cudaStream_t s);
 // x += alpha p, r -= alpha q, scal[rr] = |r|^2 with alpha = scal[num]/scal[den];
-// with b non-null also b = float(r), zpre = omega dinv b (the next V-cycle's
-// right-hand side and pre-smoothing from zero); host_rr (may be null): a
-// device-accessible pointer to pinned host memory that also receives |r|^2
+// b = float(r), zpre = omega dinv b (the next V-cycle's right-hand side and
+// pre-smoothing from zero); host_rr (may be null): a device-accessible pointer
+// to pinned host memory that also receives |r|^2
 cudaError_t launch_cg_xr_d2(long long n, void* x, void* r, const void* p, const float* q,
                             double* scal, int num, int den, int rr, double* partials,
                             unsigned* counter, float* b, float* zpre, const float* dinv,

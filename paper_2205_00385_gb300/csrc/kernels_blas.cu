@@ -1,7 +1,8 @@
 // Float64 vector kernels of the CG recursion, the CARM/PARM multi-vector
 // products and Gram-Schmidt, and small dense solves run on one block.
-// All reductions use a fixed grid of RED_BLOCKS blocks and a fixed summation
-// tree, so results do not depend on timing or on other work on the GPU.
+// All reductions use a grid fixed by the length (at most RED_BLOCKS blocks) and
+// a fixed summation tree, so results do not depend on timing or on other work
+// on the GPU.
 #include <math.h>
 
 #include "kernels.h"
@@ -12,10 +13,12 @@ __global__ void __launch_bounds__(RED_THREADS)
     k_dot(long long n, const double* __restrict__ a, const double* __restrict__ b,
           double* partials, unsigned* counter, double* out) {
   __shared__ double sh[32];
+  pdl_wait();
   double v[1] = {0.0};
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n;
        q += (long long)gridDim.x * blockDim.x)
     v[0] = fma(a[q], b[q], v[0]);
+  pdl_launch_dependents();
   block_sum<1>(v, sh);
   if (publish_partials<1>(v, partials, counter)) {
     double o[1];
@@ -30,8 +33,11 @@ __global__ void __launch_bounds__(RED_THREADS)
     k_cg_xr(long long n, double* __restrict__ x, double* __restrict__ r,
             const double* __restrict__ p, const double* __restrict__ q, double* scal, int num,
             int den, int rr, double* partials, unsigned* counter, double* host_rr) {
-  __shared__ double sh[32];
-  const double alpha = scal[num] / scal[den];
+  __shared__ double sh[32], s_alpha;
+  pdl_wait();
+  if (threadIdx.x == 0) s_alpha = scal[num] / scal[den];   // one division per block
+  __syncthreads();
+  const double alpha = s_alpha;
   double v[1] = {0.0};
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
@@ -40,6 +46,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     r[i] = ri;
     v[0] = fma(ri, ri, v[0]);
   }
+  pdl_launch_dependents();
   block_sum<1>(v, sh);
   if (publish_partials<1>(v, partials, counter)) {
     double o[1];
@@ -57,7 +64,11 @@ __global__ void __launch_bounds__(RED_THREADS)
 __global__ void __launch_bounds__(256)
     k_cg_p(long long n, double* __restrict__ p, const double* __restrict__ z,
            const double* __restrict__ scal, int num, int den) {
-  const double beta = scal[num] / scal[den];
+  __shared__ double s_beta;
+  pdl_wait();
+  if (threadIdx.x == 0) s_beta = scal[num] / scal[den];
+  __syncthreads();
+  const double beta = s_beta;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     p[i] = fma(beta, p[i], z[i]);
@@ -333,6 +344,10 @@ __global__ void k_eps(const double* scal, int rr, int f2, double* eps_dev) {
 // ---------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------
+// Blocks of the element-wise kernels and reductions: as many as have indices to
+// work on (a block without any adds a zero, so its absence changes no bits),
+// RED_BLOCKS at most.  Short vectors are bound by the reduction's last block:
+// 2,562 DOFs took 7.1 us a dot product on 608 blocks.
 static inline int vgrid(long long n) {
   long long b = (n + 255) / 256;
   if (b > RED_BLOCKS) b = RED_BLOCKS;
@@ -341,22 +356,20 @@ static inline int vgrid(long long n) {
 
 cudaError_t launch_dot(long long n, const double* a, const double* b, double* partials,
                        unsigned* counter, double* out, cudaStream_t s) {
-  k_dot<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, a, b, partials, counter, out);
-  return cudaGetLastError();
+  return launch_pdl(k_dot, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n, a, b, partials, counter,
+                    out);
 }
 
 cudaError_t launch_cg_xr(long long n, double* x, double* r, const double* p, const double* q,
                          double* scal, int num, int den, int rr, double* partials,
                          unsigned* counter, cudaStream_t s, double* host_rr) {
-  k_cg_xr<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, x, r, p, q, scal, num, den, rr, partials,
-                                             counter, host_rr);
-  return cudaGetLastError();
+  return launch_pdl(k_cg_xr, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n, x, r, p, q, scal, num, den,
+                    rr, partials, counter, host_rr);
 }
 
 cudaError_t launch_cg_p(long long n, double* p, const double* z, const double* scal, int num,
                         int den, cudaStream_t s) {
-  k_cg_p<<<vgrid(n), 256, 0, s>>>(n, p, z, scal, num, den);
-  return cudaGetLastError();
+  return launch_pdl(k_cg_p, dim3(vgrid(n)), dim3(256), 0, s, n, p, z, scal, num, den);
 }
 
 

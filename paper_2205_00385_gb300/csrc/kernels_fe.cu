@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(128)
   using TE = typename std::conditional<(sizeof(TY) > sizeof(TC)), double, TC>::type;
 
   const long long node = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
   if (node >= g.nn) return;
   const int i = (int)(node % g.nnx);
   const long long rest = node / g.nnx;
@@ -527,11 +528,11 @@ static cudaError_t run_apply(const ApplyArgs& a, cudaStream_t s) {
     for (int q = 0; q < ND * ND; ++q) ke.v[q] = TC(0);
   }
   const int th = 128;
-  k_apply<DIM, TC, TX, TY, EPI, EXPL><<<nblocks(a.g.nn, th), th, 0, s>>>(
-      a.g, a.mask, ke, static_cast<const TC*>(a.coef), static_cast<const TC*>(a.Kc),
-      static_cast<const TX*>(a.x), static_cast<TY*>(a.y), static_cast<const TX*>(a.b),
-      static_cast<const TC*>(a.dinv), TC(a.omega), TC(a.dfix), a.springs);
-  return cudaGetLastError();
+  return launch_pdl(k_apply<DIM, TC, TX, TY, EPI, EXPL>, dim3(nblocks(a.g.nn, th)), dim3(th), 0, s,
+                    a.g, a.mask, ke, static_cast<const TC*>(a.coef), static_cast<const TC*>(a.Kc),
+                    static_cast<const TX*>(a.x), static_cast<TY*>(a.y),
+                    static_cast<const TX*>(a.b), static_cast<const TC*>(a.dinv), TC(a.omega),
+                    TC(a.dfix), a.springs);
 }
 
 template <int DIM, typename TC, typename TX, typename TY, bool EXPL>

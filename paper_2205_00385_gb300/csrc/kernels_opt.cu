@@ -334,51 +334,6 @@ __device__ __forceinline__ double oc_lam_of(double s, double eta) {
   return eta == 0.5 ? 1.0 / (s * s) : pow(s, -1.0 / eta);
 }
 
-// Sums of NV double-float values per thread over the grid, finished by the
-// last block: warps reduce in double-float, then one warp per value adds the
-// warp results, and in the last block the block results, in float64 in a
-// fixed order.  Returns true in the last block, where out[] (shared) is set.
-template <int NV>
-__device__ __forceinline__ bool oc_grid_sum(const dfl (&v)[NV], double (&out)[NV],
-                                            double (&sh)[NV][OC_T / 32], double* partials,
-                                            unsigned* counter) {
-  __shared__ bool s_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    dfl x = v[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const dfl y = {__shfl_down_sync(0xffffffffu, x.h, o), __shfl_down_sync(0xffffffffu, x.l, o)};
-      x = df_add(x, y);
-    }
-    if (lane == 0) sh[q][warp] = df_to_d(x);
-  }
-  __syncthreads();
-  if (warp < NV) {
-    double t = lane < OC_T / 32 ? sh[warp][lane] : 0.0;
-#pragma unroll
-    for (int o = OC_T / 64; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) partials[(size_t)blockIdx.x * NV + warp] = t;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return false;
-  __threadfence();
-  if (warp < NV) {
-    double t = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) t += partials[(size_t)b * NV + warp];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) out[warp] = t;
-  }
-  if (threadIdx.x == 0) *counter = 0u;
-  __syncthreads();
-  return true;
-}
-
 // bracket within its final width (also when both ends are 0)
 __device__ __forceinline__ bool oc_done(double l1, double l2) {
   return !((l2 - l1) > 1e-13 * (l1 + l2));
@@ -466,7 +421,7 @@ __global__ void __launch_bounds__(OC_T)
   }
 #pragma unroll
   for (int q = 0; q < 3; ++q) v[q] = df_norm(v[q]);
-  if (!oc_grid_sum<3>(v, tot, sh, partials, counter) || threadIdx.x >= 32) return;
+  if (!grid_sum_df(v, sh, tot, partials, counter) || threadIdx.x >= 32) return;
   const double l0 = oc_lam_of(target / tot[0], eta);
   const double l1 = tot[1] > target && tot[2] > target ? OC_LAM_MAX : 0.0;
   const double l2 = tot[1] > target ? OC_LAM_MAX : 0.0;
@@ -506,7 +461,7 @@ __global__ void __launch_bounds__(OC_T, 2)
 #pragma unroll
   for (int j = 0; j < OC_NP; ++j) v[j] = df_norm(v[j]);
   pdl_launch_dependents();
-  if (!oc_grid_sum<OC_NP>(v, tot, sh, partials, counter) || threadIdx.x >= 32) return;
+  if (!grid_sum_df(v, sh, tot, partials, counter) || threadIdx.x >= 32) return;
   // the volume decreases with lambda: keep the last point above target and
   // the first at or below it
   int k = 0;

@@ -9,6 +9,7 @@
 // need no conversion and the FP64 pipe is left idle.  Reductions use a
 // fixed grid and fixed summation orders, so results do not depend on
 // scheduling.
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -526,143 +527,180 @@ __global__ void k_gs_record(const double* scal, int n0, int n1, double tol, int 
 // works on the float32 shadow p32 -> q32 and the V-cycle returns z32.
 // alpha and beta are formed once per block from the float64 scalars.
 // ---------------------------------------------------------------------------
-// The three passes below keep four indices per thread in flight (their
-// loads are issued before any of them is used), enough outstanding bytes to
-// stream at the copy bandwidth with one resident grid.
-constexpr int CG_U = 4;
+// Grids cover short vectors once (a reduction's last block bounds those: at
+// 27 k DOFs 608 blocks took 7.5 us a dot product and 9.6 us an update), with
+// at most RED_BLOCKS blocks.  In the two updates a thread takes two
+// neighbouring indices per 16- or 8-byte load (the vectors are the workspace's
+// own, 256-byte aligned; a last odd index goes to one thread): at n = 5.4 M
+// 45.8 and 17.0 us instead of 46.5 and 19.0, which is the copy bandwidth.
+constexpr int VEC_T = 256, VEC_W = VEC_T / 32;
 
-// out = sum_k a[k] b[k], a pairs, b float32.  Twelve bytes per index, so
-// eight indices per thread are kept in flight.
+struct Pair2 {
+  dfl v[2];
+};
+__device__ __forceinline__ Pair2 ld_pair2(const float2* p, long long q) {
+  const float4 t = reinterpret_cast<const float4*>(p)[q];
+  return {{{t.x, t.y}, {t.z, t.w}}};
+}
+__device__ __forceinline__ void st_pair2(float2* p, long long q, const Pair2& a) {
+  reinterpret_cast<float4*>(p)[q] = make_float4(a.v[0].h, a.v[0].l, a.v[1].h, a.v[1].l);
+}
+__device__ __forceinline__ float2 ld_two(const float* p, long long q) {
+  return reinterpret_cast<const float2*>(p)[q];
+}
+
+// body(q) for the pairs of indices (2 q, 2 q + 1) below n of this thread, U at
+// a time (load(q, u) first for all of them, then use(q, u)); odd(k) for a last
+// odd index.
+template <int U, typename Load, typename Use, typename Odd>
+__device__ __forceinline__ void pair_loop2(long long n, Load load, Use use, Odd odd) {
+  const long long m = n >> 1, stride = (long long)gridDim.x * VEC_T;
+  long long q = (long long)blockIdx.x * VEC_T + threadIdx.x;
+  if (q == 0 && (n & 1)) odd(n - 1);
+  for (; q + (U - 1) * stride < m; q += U * stride) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) load(q + u * stride, u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) use(q + u * stride, u);
+  }
+  for (; q < m; q += stride) {
+    load(q, 0);
+    use(q, 0);
+  }
+}
+
+// out = sum_k a[k] b[k], a pairs, b float32.  Twelve bytes per index, one index
+// per load and eight in flight: two indices per load measured 19 us instead of
+// 17 at n = 5.4 M.
 constexpr int DOT_U = 8;
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(VEC_T)
     k_dot_d2f(long long n, const float2* __restrict__ a, const float* __restrict__ b,
               double* partials, unsigned* counter, double* out) {
-  using Rg = Ar<float2>;
-  __shared__ double sh[32];
+  __shared__ double sh[1][VEC_W], tot[1];
   pdl_wait();
-  dfl v[2] = {Rg::zero(), Rg::zero()};
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  dfl v[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  const long long stride = (long long)gridDim.x * VEC_T;
+  long long k = (long long)blockIdx.x * VEC_T + threadIdx.x;
   for (; k + (DOT_U - 1) * stride < n; k += DOT_U * stride) {
     dfl av[DOT_U];
     float bv[DOT_U];
 #pragma unroll
     for (int u = 0; u < DOT_U; ++u) {
-      av[u] = Rg::ld(a, k + u * stride);
+      av[u] = ld_df(a, k + u * stride);
       bv[u] = b[k + u * stride];
     }
 #pragma unroll
     for (int u = 0; u < DOT_U; ++u) df_dot_acc(v[u & 1], av[u], dfl{bv[u], 0.f});
   }
-  for (; k < n; k += stride) df_dot_acc(v[0], Rg::ld(a, k), dfl{b[k], 0.f});
-  reduce_to<float2>(df_add(df_norm(v[0]), df_norm(v[1])), out, partials, counter, sh);
+  for (; k < n; k += stride) df_dot_acc(v[0], ld_df(a, k), dfl{b[k], 0.f});
   pdl_launch_dependents();
+  const dfl w[1] = {df_add(df_norm(v[0]), df_norm(v[1]))};
+  if (grid_sum_df(w, sh, tot, partials, counter) && threadIdx.x == 0) *out = tot[0];
 }
 
 // alpha = scal[num] / scal[den]; x += alpha p; r -= alpha q; scal[rr] = |r|^2.
-// With b non-null it also starts the next V-cycle: b = r rounded to float32
-// and zpre = omega dinv b (its pre-smoothing from a zero guess), the values
-// the V-cycle's first kernel would compute.
+// It also starts the next V-cycle: b = r rounded to float32 and
+// zpre = omega dinv b (its pre-smoothing from a zero guess), the values the
+// V-cycle's first kernel would compute.
 // With host_rr set, |r|^2 is also written there (pinned host memory mapped
 // into the device's address space), so the host reads it after an event on
 // the stream without a copy between this kernel and the next.
-template <bool PRE>
-__global__ void __launch_bounds__(RED_THREADS)
+constexpr int CG_U = 2;
+__global__ void __launch_bounds__(VEC_T)
     k_cg_xr_d2(long long n, float2* __restrict__ x, float2* __restrict__ r,
                const float2* __restrict__ p, const float* __restrict__ q, double* scal, int num,
                int den, int rr, double* partials, unsigned* counter, float* __restrict__ b,
                float* __restrict__ zpre, const float* __restrict__ dinv, float omega,
                double* host_rr) {
   using Rg = Ar<float2>;
-  __shared__ double sh[32];
-  __shared__ double s_alpha;
+  __shared__ double sh[1][VEC_W], tot[1];
+  __shared__ dfl s_alpha;
   pdl_wait();
-  if (threadIdx.x == 0) s_alpha = scal[num] / scal[den];
+  if (threadIdx.x == 0) s_alpha = split_d(scal[num] / scal[den]);
   __syncthreads();
-  const dfl al = split_d(s_alpha), mal = {-al.h, -al.l};
-  dfl v[2] = {Rg::zero(), Rg::zero()};
-  auto step = [&](long long kk, dfl xk, dfl pk, dfl rk0, float qk, float dk, dfl& acc) {
-    Rg::st(x, kk, df_fma(al, pk, xk));
-    const dfl rk = df_add(Rg::mulf(mal, qk), rk0);
-    Rg::st(r, kk, rk);
+  const dfl al = s_alpha, mal = {-al.h, -al.l};
+  dfl v[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  // one index: updates xk and rk, returns b
+  auto step = [&](dfl& xk, dfl& rk, dfl pk, float qk, dfl& acc) {
+    xk = df_fma(al, pk, xk);
+    rk = df_add(Rg::mulf(mal, qk), rk);
     df_dot_acc(acc, rk, rk);
-    if (PRE) {
-      const float bv = __fadd_rn(rk.h, rk.l);
-      b[kk] = bv;
-      zpre[kk] = omega * dk * bv;
-    }
+    return __fadd_rn(rk.h, rk.l);
   };
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  for (; k + (CG_U - 1) * stride < n; k += CG_U * stride) {
-    dfl xv[CG_U], pv[CG_U], rv[CG_U];
-    float qv[CG_U], dv[CG_U];
-#pragma unroll
-    for (int u = 0; u < CG_U; ++u) {
-      const long long kk = k + u * stride;
-      xv[u] = Rg::ld(x, kk);
-      pv[u] = Rg::ld(p, kk);
-      rv[u] = Rg::ld(r, kk);
-      qv[u] = q[kk];
-      dv[u] = PRE ? dinv[kk] : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < CG_U; ++u)
-      step(k + u * stride, xv[u], pv[u], rv[u], qv[u], dv[u], v[u & 1]);
-  }
-  for (; k < n; k += stride)
-    step(k, Rg::ld(x, k), Rg::ld(p, k), Rg::ld(r, k), q[k], PRE ? dinv[k] : 0.f, v[0]);
-  {
-    // reduce_to's sum, with the second destination
-    typename Ar<float2>::T vv[1] = {df_add(df_norm(v[0]), df_norm(v[1]))};
-    double o1[1];
-    block_sum_v<float2, 1>(vv, o1, sh);
-    if (publish_partials<1>(o1, partials, counter)) {
-      double o[1];
-      finish_sum<1>(partials, counter, o, sh);
-      if (threadIdx.x == 0) {
-        scal[rr] = o[0];
-        if (host_rr) {
-          *reinterpret_cast<volatile double*>(host_rr) = o[0];
-          __threadfence_system();
-        }
-      }
-    }
-  }
+  Pair2 xv[CG_U], rv[CG_U], pv[CG_U];
+  float2 qv[CG_U], dv[CG_U];
+  pair_loop2<CG_U>(
+      n,
+      [&](long long k, int u) {
+        xv[u] = ld_pair2(x, k);
+        rv[u] = ld_pair2(r, k);
+        pv[u] = ld_pair2(p, k);
+        qv[u] = ld_two(q, k);
+        dv[u] = ld_two(dinv, k);
+      },
+      [&](long long k, int u) {
+        const float b0 = step(xv[u].v[0], rv[u].v[0], pv[u].v[0], qv[u].x, v[0]);
+        const float b1 = step(xv[u].v[1], rv[u].v[1], pv[u].v[1], qv[u].y, v[1]);
+        st_pair2(x, k, xv[u]);
+        st_pair2(r, k, rv[u]);
+        reinterpret_cast<float2*>(b)[k] = make_float2(b0, b1);
+        reinterpret_cast<float2*>(zpre)[k] =
+            make_float2(omega * dv[u].x * b0, omega * dv[u].y * b1);
+      },
+      [&](long long k) {
+        dfl xk = ld_df(x, k), rk = ld_df(r, k);
+        const float bk = step(xk, rk, ld_df(p, k), q[k], v[0]);
+        st_df(x, k, xk);
+        st_df(r, k, rk);
+        b[k] = bk;
+        zpre[k] = omega * dinv[k] * bk;
+      });
   pdl_launch_dependents();
+  const dfl w[1] = {df_add(df_norm(v[0]), df_norm(v[1]))};
+  if (grid_sum_df(w, sh, tot, partials, counter) && threadIdx.x == 0) {
+    scal[rr] = tot[0];
+    if (host_rr) {
+      *reinterpret_cast<volatile double*>(host_rr) = tot[0];
+      __threadfence_system();
+    }
+  }
 }
 
 // p = z + beta p (beta = scal[num]/scal[den], or p = z when num < 0);
 // p32 = p rounded to float32
-__global__ void __launch_bounds__(256)
+constexpr int CGP_U = 4;
+__global__ void __launch_bounds__(VEC_T)
     k_cg_p_d2(long long n, float2* __restrict__ p, float* __restrict__ p32,
               const float* __restrict__ z, const double* __restrict__ scal, int num, int den) {
-  using Rg = Ar<float2>;
-  __shared__ double s_beta;
+  __shared__ dfl s_beta;
   pdl_wait();
-  if (threadIdx.x == 0) s_beta = num >= 0 ? scal[num] / scal[den] : 0.0;
+  const bool restart = num < 0;
+  if (threadIdx.x == 0) s_beta = split_d(restart ? 0.0 : scal[num] / scal[den]);
   __syncthreads();
-  const dfl be = split_d(s_beta);
-  auto step = [&](long long kk, float zv, dfl pold) {
+  const dfl be = s_beta;
+  auto step = [&](float zv, dfl pold) {
     const dfl zk = {zv, 0.f};
-    const dfl pk = num >= 0 ? df_add(df_mul(be, pold), zk) : zk;
-    Rg::st(p, kk, pk);
-    p32[kk] = __fadd_rn(pk.h, pk.l);
+    return restart ? zk : df_add(df_mul(be, pold), zk);
   };
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  for (; k + (CG_U - 1) * stride < n; k += CG_U * stride) {
-    float zv[CG_U];
-    dfl pv[CG_U];
-#pragma unroll
-    for (int u = 0; u < CG_U; ++u) {
-      zv[u] = z[k + u * stride];
-      pv[u] = num >= 0 ? Rg::ld(p, k + u * stride) : Rg::zero();
-    }
-#pragma unroll
-    for (int u = 0; u < CG_U; ++u) step(k + u * stride, zv[u], pv[u]);
-  }
-  for (; k < n; k += stride) step(k, z[k], num >= 0 ? Rg::ld(p, k) : Rg::zero());
+  Pair2 pv[CGP_U];
+  float2 zv[CGP_U];
+  pair_loop2<CGP_U>(
+      n,
+      [&](long long k, int u) {
+        if (!restart) pv[u] = ld_pair2(p, k);
+        zv[u] = ld_two(z, k);
+      },
+      [&](long long k, int u) {
+        const Pair2 o = {{step(zv[u].x, pv[u].v[0]), step(zv[u].y, pv[u].v[1])}};
+        st_pair2(p, k, o);
+        reinterpret_cast<float2*>(p32)[k] =
+            make_float2(__fadd_rn(o.v[0].h, o.v[0].l), __fadd_rn(o.v[1].h, o.v[1].l));
+      },
+      [&](long long k) {
+        const dfl o = step(z[k], restart ? dfl{0.f, 0.f} : ld_df(p, k));
+        st_df(p, k, o);
+        p32[k] = __fadd_rn(o.h, o.l);
+      });
   pdl_launch_dependents();
 }
 
@@ -901,28 +939,29 @@ cudaError_t launch_combine_multi(long long n, int vt, const void* Q, int kq, con
   return cudaGetLastError();
 }
 
+static dim3 pair2_grid(long long n, int per_thread) {
+  const long long b = (n + 2LL * per_thread * VEC_T - 1) / (2LL * per_thread * VEC_T);
+  return dim3((unsigned)std::min<long long>(std::max<long long>(b, 1), RED_BLOCKS));
+}
+
 cudaError_t launch_dot_d2f(long long n, const void* a, const float* b, double* partials,
                            unsigned* counter, double* out, cudaStream_t s) {
-  return launch_pdl(k_dot_d2f, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n, (const float2*)a, b,
-                    partials, counter, out);
+  return launch_pdl(k_dot_d2f, pair2_grid(n, 1), dim3(VEC_T), 0, s, n, (const float2*)a, b, partials,
+                    counter, out);
 }
 
 cudaError_t launch_cg_xr_d2(long long n, void* x, void* r, const void* p, const float* q,
                             double* scal, int num, int den, int rr, double* partials,
                             unsigned* counter, float* b, float* zpre, const float* dinv,
                             double omega, cudaStream_t s, double* host_rr) {
-  if (b)
-    return launch_pdl(k_cg_xr_d2<true>, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n, (float2*)x,
-                      (float2*)r, (const float2*)p, q, scal, num, den, rr, partials, counter, b,
-                      zpre, dinv, (float)omega, host_rr);
-  return launch_pdl(k_cg_xr_d2<false>, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n, (float2*)x,
-                    (float2*)r, (const float2*)p, q, scal, num, den, rr, partials, counter,
-                    (float*)nullptr, (float*)nullptr, (const float*)nullptr, 0.f, host_rr);
+  return launch_pdl(k_cg_xr_d2, pair2_grid(n, 1), dim3(VEC_T), 0, s, n, (float2*)x, (float2*)r,
+                    (const float2*)p, q, scal, num, den, rr, partials, counter, b, zpre, dinv,
+                    (float)omega, host_rr);
 }
 
 cudaError_t launch_cg_p_d2(long long n, void* p, float* p32, const float* z, const double* scal,
                            int num, int den, cudaStream_t s) {
-  return launch_pdl(k_cg_p_d2, dim3(vgrid(n)), dim3(256), 0, s, n, (float2*)p, p32, z, scal, num,
+  return launch_pdl(k_cg_p_d2, pair2_grid(n, 1), dim3(VEC_T), 0, s, n, (float2*)p, p32, z, scal, num,
                     den);
 }
 

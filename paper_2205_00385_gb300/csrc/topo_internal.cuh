@@ -255,6 +255,41 @@ __device__ __forceinline__ void finish_sum(const double* partials, unsigned* cou
   if (threadIdx.x == 0) *counter = 0u;
 }
 
+// Sums of NV values over the grid from each warp's values sh[q][warp]: one
+// warp per value adds the block's, and in the last block to arrive the
+// blocks', in float64 in a fixed order.  Returns true in the last block, where
+// out[] (shared) is set.  Needs at least NV warps per block.
+template <int NV, int NW>
+__device__ __forceinline__ bool grid_sum(double (&sh)[NV][NW], double (&out)[NV],
+                                         double* partials, unsigned* counter) {
+  static_assert(NV <= NW && (NW & (NW - 1)) == 0 && NW <= 32, "one warp per value");
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __syncthreads();
+  if (warp < NV) {
+    double t = lane < NW ? sh[warp][lane] : 0.0;
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) partials[(size_t)blockIdx.x * NV + warp] = t;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  if (warp < NV) {
+    double t = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += partials[(size_t)b * NV + warp];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) out[warp] = t;
+  }
+  if (threadIdx.x == 0) *counter = 0u;
+  __syncthreads();
+  return true;
+}
+
 template <int NV>
 __device__ __forceinline__ void finish_max(const double* partials, unsigned* counter,
                                            double (&out)[NV], double* sh) {
