@@ -238,6 +238,11 @@ cudaError_t launch_gs_accept(long long n, int vt, void* R, int src, const double
 // Y[:, j] = sum_{i < kq} U[i + MAXB j] Q[:, i] for j < k <= kq (Y != Q)
 cudaError_t launch_combine_multi(long long n, int vt, const void* Q, int kq, const double* U,
                                  int k, void* Y, cudaStream_t s);
+// 2D mixed CG: q = K p (p pairs, zero on the fixed DOFs; q float32) in
+// double-float, *pq = p . q (kernels_df.cu); ke64: host pointer to KE
+cudaError_t launch_cg_q2_df(const GridP& g, const uint8_t* mask, const double* ke64,
+                            const double* coef, const void* p, float* q, const Springs& sp,
+                            double* partials, unsigned* counter, double* pq, cudaStream_t s);
 // mixed-path CG (pairs x, r, p; float32 shadows p32 -> q32 and z32; vectors of
 // the workspace, 16-byte aligned): out = a . b
 cudaError_t launch_dot_d2f(long long n, const void* a, const float* b, double* partials,

@@ -8,6 +8,7 @@
 // operations, so the FP64 pipe only sees the final additions of the
 // epilogue.  The structure (element columns streamed in z, owner-computes
 // node sums in shared memory, Walsh blocks) is that of k_apply3_col.
+#include <algorithm>
 #include <type_traits>
 
 #include "dfmath.cuh"
@@ -159,6 +160,102 @@ __global__ void __launch_bounds__(DX * DY)
     }
     buf ^= 1;
   }
+}
+
+// ---------------------------------------------------------------------------
+// 2D: q = K p of the mixed CG with p in pairs, in double-float arithmetic,
+// rounded to float32 at the end, and p . q of that q.  On a smooth direction
+// K p is smaller than K's entries times p by (element size / wave length)^2,
+// 2e-6 on a 640-element span, so the float32 product of p rounded to float32
+// (6e-8) is off by percents there and the CG takes up to twice the iterations.
+// One thread per node gathers its nine nodes (16 bytes each) and forms its two
+// rows of the four elements around it, each row a Dot2 sum.  About 950 FP32
+// instructions per node; the direction is zero on the fixed DOFs (a fixed row's
+// product is 0).  Twelve solves at 640 x 320 to 1e-6: 1001 iterations in 129 ms
+// with the float32 product, 738 in 76 ms with this one (float64: 726); at
+// 320 x 160 614 in 67 ms and 307 in 25 ms.
+// ---------------------------------------------------------------------------
+struct DfKe2 {
+  float2 v[8][8];
+};
+constexpr int D2_T = 256, D2_BLOCKS = 8 * 152;
+
+__global__ void __launch_bounds__(D2_T)
+    k_cg_q2_df(GridP g, const uint8_t* __restrict__ mask, DfKe2 ke,
+               const double* __restrict__ coef, const float2* __restrict__ p,
+               float* __restrict__ q, Springs sp, double* partials, unsigned* counter,
+               double* pq) {
+  __shared__ double sh[1][D2_T / 32], tot[1];
+  pdl_wait();
+  dfl dot[1] = {{0.f, 0.f}};
+  for (long long node = (long long)blockIdx.x * D2_T + threadIdx.x; node < g.nn;
+       node += (long long)gridDim.x * D2_T) {
+    const int i = (int)(node % g.nnx), j = (int)(node / g.nnx);
+    // clamped neighbours: outside the grid their elements' moduli are 0
+    float4 x[3][3];
+    dfl E[2][2];
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int ii = min(max(i + a - 1, 0), g.nnx - 1), jj = min(max(j + b - 1, 0), g.nny - 1);
+        x[b][a] = reinterpret_cast<const float4*>(p)[ii + (long long)g.nnx * jj];
+      }
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const int ei = i - 1 + a, ej = j - 1 + b;
+        const bool in = ei >= 0 && ei < g.nx && ej >= 0 && ej < g.ny;
+        E[b][a] = in ? split_d(coef[ei + (long long)g.nx * ej]) : dfl{0.f, 0.f};
+      }
+    dfl acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const int corner = (1 - a) + 2 * (1 - b);   // of this node in element (a, b)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          dfl s = {0.f, 0.f};
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const float4 u = x[b + (m >> 1)][a + (m & 1)];
+            const float2 k0 = ke.v[2 * corner + c][2 * m], k1 = ke.v[2 * corner + c][2 * m + 1];
+            df_dot_acc(s, {k0.x, k0.y}, {u.x, u.y});
+            df_dot_acc(s, {k1.x, k1.y}, {u.z, u.w});
+          }
+          acc[c] = df_fma(E[b][a], df_norm(s), acc[c]);
+        }
+      }
+    const unsigned m = mask[node];
+    const dfl own[2] = {{x[1][1].x, x[1][1].y}, {x[1][1].z, x[1][1].w}};
+    float out[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      for (int t = 0; t < sp.n; ++t)
+        if (sp.dof[t] == 2 * node + c) acc[c] = df_fma(split_d(sp.k[t]), own[c], acc[c]);
+      out[c] = ((m >> c) & 1u) ? 0.f : __fadd_rn(acc[c].h, acc[c].l);
+      df_dot_acc(dot[0], own[c], {out[c], 0.f});
+    }
+    reinterpret_cast<float2*>(q)[node] = make_float2(out[0], out[1]);
+  }
+  pdl_launch_dependents();
+  dot[0] = df_norm(dot[0]);
+  if (grid_sum_df(dot, sh, tot, partials, counter) && threadIdx.x == 0) *pq = tot[0];
+}
+
+cudaError_t launch_cg_q2_df(const GridP& g, const uint8_t* mask, const double* ke64,
+                            const double* coef, const void* p, float* q, const Springs& sp,
+                            double* partials, unsigned* counter, double* pq, cudaStream_t s) {
+  DfKe2 ke;
+  for (int e = 0; e < 64; ++e) {
+    const float h = (float)ke64[e];
+    (&ke.v[0][0])[e] = make_float2(h, (float)(ke64[e] - (double)h));
+  }
+  const int blocks = std::min(nblocks(g.nn, D2_T), D2_BLOCKS);
+  return launch_pdl(k_cg_q2_df, dim3(blocks), dim3(D2_T), 0, s, g, mask, ke, coef, (const float2*)p,
+                    q, sp, partials, counter, pq);
 }
 
 bool df_blocks_ok(const double* wht64) {

@@ -1080,21 +1080,6 @@ static to_status apply_op(to_ctx* c, int op, int prec, const double* x, double* 
 static int vt(const to_ctx* c) { return c->mixed ? V_DF2 : V_F64; }
 static int vt_code(const to_ctx* c) { return c->mixed ? T_D2 : T_F64; }
 
-// y = op(x) in the context's apply precision, x and y in vector storage:
-// float64 on the FP64 path; float32 through the shadows p32 -> q32 (the
-// solver's float32 operator) on the mixed path
-static to_status apply_vec(to_ctx* c, int op, const double* x, double* y) {
-  if (!c->mixed)
-    return run_op(c, fine_args(c, op, T_F64, T_F64, T_F64, x, y, nullptr, nullptr, EPI_APPLY),
-                  "apply");
-  LAUNCH(c, launch_convert(T_D2, T_F32, c->n, x, c->p32, c->stream), "round x");
-  to_status st = run_op(c, fine_args(c, op, T_F32, T_F32, T_F32, c->p32, c->q32, nullptr,
-                                     nullptr, EPI_APPLY), "apply");
-  if (st != TO_OK) return st;
-  LAUNCH(c, launch_convert(T_F32, T_D2, c->n, c->q32, y, c->stream), "widen y");
-  return TO_OK;
-}
-
 // float64-accurate y = op(x) (EPI_APPLY) or y = f - op(x) (EPI_RESID), x
 // and y in vector storage: float64 operator, double-float operator on pairs,
 // or (mixed 2D) the float64 operator through float64 scratch
@@ -1252,10 +1237,11 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
     else
       LAUNCH(c, launch_copy(n, c->z, c->p, s), "p = z");
     int cur = S_RZ0, nxt = S_RZ1;
-    // Precision escalation (mixed path): q = K p in float32 carries ~1e-4
-    // relative error on smooth search directions (K cancels by 1e3-1e4
-    // there), and on some designs CG stagnates on it, the recursive and
-    // true residuals stuck together.  Healthy convergence gains >= 10x in
+    // Precision escalation (mixed path, 3D; in 2D, where a float32 K p loses
+    // percents on the longer spans, q is formed in double-float throughout):
+    // q = K p in float32 carries ~1e-4 relative error on smooth search
+    // directions (K cancels by 1e3-1e4 there), and on some designs CG
+    // stagnates on it, the recursive and true residuals stuck together.  Healthy convergence gains >= 10x in
     // 16 iterations; when the residual fails to halve over 16 iterations,
     // the rest of the solve forms q with the double-float operator (then
     // rounded to float32, which loses nothing to cancellation) and CG
@@ -1264,7 +1250,11 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
     double rel_window = rel;
     int it_window = 0;
     for (it = 1; it <= maxit; ++it) {
-      if (mixed && accurate_q) {
+      if (mixed && c->dim == 2) {
+        LAUNCH(c, launch_cg_q2_df(c->lv[0].g, c->lv[0].mask, c->KE64, c->E64, c->p, c->q32,
+                                  c->springs, c->partials, c->counters + C_DOT, c->scal + S_PQ, s),
+               "q = K p, pq");
+      } else if (mixed && accurate_q) {
         if ((st = apply_accurate_vec(c, TO_OP_K, c->p, c->t, EPI_APPLY)) != TO_OK) return st;
         LAUNCH(c, launch_convert(T_D2, T_F32, n, c->t, c->q32, s), "q to float32");
       } else if (mixed) {
@@ -1274,8 +1264,9 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
         if ((st = run_op(c, a, "q = K p")) != TO_OK) return st;
       }
       if (mixed) {
-        LAUNCH(c, launch_dot_d2f(n, c->p, c->q32, c->partials, c->counters + C_DOT,
-                                 c->scal + S_PQ, s), "pq");
+        if (c->dim == 3)
+          LAUNCH(c, launch_dot_d2f(n, c->p, c->q32, c->partials, c->counters + C_DOT,
+                                   c->scal + S_PQ, s), "pq");
         LAUNCH(c, launch_cg_xr_d2(n, x, c->r, c->p, c->q32, c->scal, cur, S_PQ, S_RR,
                                   c->partials, c->counters + C_UPD,
                                   static_cast<float*>(c->lv[0].b), static_cast<float*>(c->lv[0].z),
@@ -1317,7 +1308,7 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
       // (p = z).
       bool restart = false;
       bool escalate = false;
-      if (mixed && !accurate_q && it - it_window >= 16) {
+      if (mixed && c->dim == 3 && !accurate_q && it - it_window >= 16) {
         escalate = rel > 0.5 * rel_window;
         rel_window = rel;
         it_window = it;
