@@ -324,7 +324,7 @@ cudaError_t launch_apply_df(const ApplyArgs& a, cudaStream_t s) {
       a.tx == T_D2 ? (a.epi == EPI_RESID ? df_slots<EPI_RESID>() : df_slots<EPI_APPLY>()) : 0;
   if (slots > 0) {
     long long best = -1;
-    for (int c = 2; c <= a.g.nnz; ++c) {
+    for (int c = 1; c <= a.g.nnz; ++c) {
       const long long blocks = (long long)gx * gy * ((a.g.nnz + c - 1) / c);
       const long long cost = ((blocks + slots - 1) / slots) * (c + 1);
       if (best < 0 || cost < best) {

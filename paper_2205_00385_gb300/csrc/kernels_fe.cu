@@ -593,12 +593,14 @@ static cudaError_t run_col(const ApplyArgs& a, cudaStream_t s) {
   int zc = WZC;
   while (zc > 2 && (long long)gx * gy * ((a.g.nnz + zc - 1) / zc) < 2 * 152) zc /= 2;
   // level-1 Galerkin operator (latency-bound, one block per column chunk):
-  // the chunk length minimising waves x (layers + 1 recomputed)
+  // the chunk length minimising waves x (layers + 1 recomputed); on small
+  // grids single layers (a V-cycle 52 -> 49 us at 32 x 16 x 16, 70 -> 66 at
+  // 64 x 32 x 32 against chunks of two)
   const long long slots =
       (OP == OPK_GAL1 && sizeof(TC) == 4 && sizeof(TX) == 4 && sizeof(TY) == 4) ? gal1_slots<EPI>() : 0;
   if (slots > 0) {
     long long best = -1;
-    for (int c = 2; c <= WZC; ++c) {
+    for (int c = 1; c <= WZC; ++c) {
       const long long blocks = (long long)gx * gy * ((a.g.nnz + c - 1) / c);
       const long long cost = ((blocks + slots - 1) / slots) * (c + 1);
       if (best < 0 || cost < best || (cost == best && c > zc)) {

@@ -270,9 +270,11 @@ __device__ __forceinline__ bool grid_sum(double (&sh)[NV][NW], double (&out)[NV]
     double t = lane < NW ? sh[warp][lane] : 0.0;
 #pragma unroll
     for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) partials[(size_t)blockIdx.x * NV + warp] = t;
+    if (lane == 0) {
+      partials[(size_t)blockIdx.x * NV + warp] = t;
+      __threadfence();   // (the writing threads only: a fence waits for all stores of its thread)
+    }
   }
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
   __syncthreads();
