@@ -90,25 +90,33 @@ __global__ void __launch_bounds__(256) k_scale_inv_sqrt(long long n, double* __r
 }
 
 // ---------------------------------------------------------------------------
-// Small dense float64 kernels (m <= 16), one thread does the work.
+// Small dense float64 kernels (m <= 16), one warp.  They are chains of float64
+// divisions and sums, so what is independent runs on lanes of its own: the
+// rows of a column of the factor, the columns of an inverse (m = 10: 164 us for
+// the inverse on one thread).
 // ---------------------------------------------------------------------------
+// Cholesky factor of the symmetrised A into shared L (column-major, zero above
+// the diagonal); false when a pivot is not positive.  Lane i owns row i.
 __device__ bool chol_small(int m, const double* A, double* L) {
-  for (int i = 0; i < m * m; ++i) L[i] = 0.0;
+  const int i = threadIdx.x & 31;
+  for (int q = i; q < m * m; q += 32) L[q] = 0.0;
+  __syncwarp();
   for (int j = 0; j < m; ++j) {
-    double d = 0.5 * (A[j + m * j] + A[j + m * j]);
-    for (int k = 0; k < j; ++k) d -= L[j + m * k] * L[j + m * k];
+    double s = 0.0;
+    if (i >= j && i < m) {
+      s = 0.5 * (A[i + m * j] + A[j + m * i]);
+      for (int k = 0; k < j; ++k) s -= L[i + m * k] * L[j + m * k];
+    }
+    const double d = __shfl_sync(0xffffffffu, s, j);
     if (!(d > 0.0)) return false;
     const double ljj = sqrt(d);
-    L[j + m * j] = ljj;
-    for (int i = j + 1; i < m; ++i) {
-      double s = 0.5 * (A[i + m * j] + A[j + m * i]);
-      for (int k = 0; k < j; ++k) s -= L[i + m * k] * L[j + m * k];
-      L[i + m * j] = s / ljj;
-    }
+    if (i >= j && i < m) L[i + m * j] = i == j ? ljj : s / ljj;
+    __syncwarp();
   }
   return true;
 }
 
+// x = (L L^T)^{-1} b by one thread
 __device__ void chol_solve_small(int m, const double* L, const double* b, double* x) {
   double y[MAXB];
   for (int i = 0; i < m; ++i) {
@@ -168,18 +176,19 @@ __device__ void jacobi_eigen(int m, double* A, double* w, double* V) {
 // eigen-pseudo-inverse with relative cutoff 1e-14.
 __global__ void k_small_spd_inverse(int mmax, const int* m_dev, const double* A, double* Ainv,
                                     int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (blockIdx.x != 0) return;
   const int m = m_dev ? min(*m_dev, mmax) : mmax;
-  double L[MAXB * MAXB];
+  __shared__ double L[MAXB * MAXB];
   if (chol_small(m, A, L)) {
+    const int j = threadIdx.x;
+    if (j >= m) return;
     double e[MAXB], col[MAXB];
-    for (int j = 0; j < m; ++j) {
-      for (int i = 0; i < m; ++i) e[i] = (i == j) ? 1.0 : 0.0;
-      chol_solve_small(m, L, e, col);
-      for (int i = 0; i < m; ++i) Ainv[i + m * j] = col[i];
-    }
+    for (int i = 0; i < m; ++i) e[i] = (i == j) ? 1.0 : 0.0;
+    chol_solve_small(m, L, e, col);
+    for (int i = 0; i < m; ++i) Ainv[i + m * j] = col[i];
     return;
   }
+  if (threadIdx.x != 0) return;
   double S[MAXB * MAXB], V[MAXB * MAXB], w[MAXB];
   for (int j = 0; j < m; ++j)
     for (int i = 0; i < m; ++i) S[i + m * j] = 0.5 * (A[i + m * j] + A[j + m * i]);
@@ -196,24 +205,24 @@ __global__ void k_small_spd_inverse(int mmax, const int* m_dev, const double* A,
   (void)status;
 }
 
-// y = sign * A x (A column-major m x m)
+// y = sign * A x (A column-major m x m), a row per lane
 __global__ void k_small_matvec(int mmax, const int* m_dev, const double* A, const double* x,
                                double* y, double sign) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int m = m_dev ? min(*m_dev, mmax) : mmax;
-  for (int i = 0; i < m; ++i) {
-    double s = 0.0;
-    for (int k = 0; k < m; ++k) s += A[i + m * k] * x[k];
-    y[i] = sign * s;
-  }
+  const int m = m_dev ? min(*m_dev, mmax) : mmax, i = threadIdx.x;
+  if (i >= m || blockIdx.x != 0) return;
+  double s = 0.0;
+  for (int k = 0; k < m; ++k) s += A[i + m * k] * x[k];
+  y[i] = sign * s;
 }
 
 __global__ void k_small_chol_solve(int mmax, const int* m_dev, const double* A, const double* b,
                                    double* x, int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (blockIdx.x != 0) return;
   const int m = m_dev ? min(*m_dev, mmax) : mmax;
-  double L[MAXB * MAXB];
-  if (!chol_small(m, A, L)) {
+  __shared__ double L[MAXB * MAXB];
+  const bool spd = chol_small(m, A, L);
+  if (threadIdx.x != 0) return;
+  if (!spd) {
     // fall back to the pseudo-inverse so that a result is still produced
     double S[MAXB * MAXB], V[MAXB * MAXB], w[MAXB];
     for (int j = 0; j < m; ++j)

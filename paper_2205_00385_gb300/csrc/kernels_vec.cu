@@ -70,45 +70,28 @@ __device__ __forceinline__ void st_any(double* p, long long i, double v) { p[i] 
 __device__ __forceinline__ void st_any(double* p, long long i, dfl v) { p[i] = df_to_d(v); }
 __device__ __forceinline__ void st_any(float2* p, long long i, dfl v) { p[i] = make_float2(v.h, v.l); }
 
-// Block sum of NV per-thread values: warps reduce in the storage's
-// arithmetic, lane 0 widens once, warp 0 adds the warp results in float64
-// in warp order.  Valid in thread 0.
-template <typename S, int NV>
-__device__ __forceinline__ void block_sum_v(typename Ar<S>::T (&v)[NV], double (&out)[NV],
-                                            double* sh /* >= NV*32 */) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// grid_sum of NV per-thread values; warps reduce in the storage's arithmetic
+template <typename S, int NV, int NW>
+__device__ __forceinline__ bool grid_sum_v(const typename Ar<S>::T (&v)[NV], double (&sh)[NV][NW],
+                                           double (&out)[NV], double* partials,
+                                           unsigned* counter) {
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
     typename Ar<S>::T x = v[q];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x = Ar<S>::add(x, Ar<S>::shfl_down(x, o));
-    if (lane == 0) sh[q * 32 + warp] = Ar<S>::to_d(x);
+    if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = Ar<S>::to_d(x);
   }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      double s = lane < nw ? sh[q * 32 + lane] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      out[q] = s;
-    }
-  }
-  __syncthreads();
+  return grid_sum<NV, NW>(sh, out, partials, counter);
 }
 
 // single-value reduction finished by the last block: *out = sum
 template <typename S>
 __device__ __forceinline__ void reduce_to(typename Ar<S>::T v, double* out, double* partials,
-                                          unsigned* counter, double* sh) {
-  typename Ar<S>::T vv[1] = {v};
-  double o1[1];
-  block_sum_v<S, 1>(vv, o1, sh);
-  if (publish_partials<1>(o1, partials, counter)) {
-    double o[1];
-    finish_sum<1>(partials, counter, o, sh);
-    if (threadIdx.x == 0) *out = o[0];
-  }
+                                          unsigned* counter) {
+  __shared__ double sh[1][RED_THREADS / 32], tot[1];
+  const typename Ar<S>::T vv[1] = {v};
+  if (grid_sum_v<S>(vv, sh, tot, partials, counter) && threadIdx.x == 0) *out = tot[0];
 }
 
 #define GRID_LOOP(k, n)                                                 \
@@ -123,7 +106,6 @@ __global__ void __launch_bounds__(RED_THREADS)
     k_vdot(long long n, const S* __restrict__ a, const S* __restrict__ b, double* partials,
            unsigned* counter, double* out) {
   using A = Ar<S>;
-  __shared__ double sh[32];
   typename A::T v[2] = {A::zero(), A::zero()};
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -138,7 +120,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     for (int u = 0; u < 4; ++u) A::dacc(v[u & 1], av[u], bv[u]);
   }
   for (; k < n; k += stride) A::dacc(v[0], A::ld(a, k), A::ld(b, k));
-  reduce_to<S>(A::add(A::dfin(v[0]), A::dfin(v[1])), out, partials, counter, sh);
+  reduce_to<S>(A::add(A::dfin(v[0]), A::dfin(v[1])), out, partials, counter);
 }
 
 __global__ void __launch_bounds__(256) k_split(long long n, const double* __restrict__ in,
@@ -297,13 +279,30 @@ __global__ void __launch_bounds__(MD_CH)
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int e = t; e < np; e += MD_CH) {
-    const int i = e % ma, j = e / ma;
-    if (sym && i > j) continue;
+  // the blocks' sums: with few entries several threads share one, each an
+  // interleaved part of the blocks
+  const int ng = np > 0 && np <= MD_CH / 2 ? MD_CH / np : 1;
+  for (int e0 = 0; e0 < np; e0 += MD_CH) {
+    const int e = ng > 1 ? t % np : e0 + t, gi = ng > 1 ? t / np : 0;
+    const int i = e < np ? e % ma : 0, j = e < np ? e / ma : 0;
+    const bool mine = e < np && gi < ng && !(sym && i > j);
     double sum = 0.0;
-    for (int bl = 0; bl < (int)gridDim.x; ++bl) sum += partials[(size_t)bl * (MAXB * MAXB) + e];
-    G[i + (size_t)ldg * j] = sum;
-    if (sym) G[j + (size_t)ldg * i] = sum;
+    if (mine) {
+#pragma unroll 8
+      for (int bl = gi; bl < (int)gridDim.x; bl += ng)
+        sum += partials[(size_t)bl * (MAXB * MAXB) + e];
+    }
+    if (ng > 1) {
+      __syncthreads();
+      red[t] = sum;
+      __syncthreads();
+      if (gi == 0)
+        for (int u = 1; u < ng; ++u) sum += red[u * np + e];
+    }
+    if (mine && gi == 0) {
+      G[i + (size_t)ldg * j] = sum;
+      if (sym) G[j + (size_t)ldg * i] = sum;
+    }
   }
   if (t == 0) *counter = 0u;
 }
@@ -360,10 +359,11 @@ __global__ void __launch_bounds__(32 * MAXB)
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if ((int)threadIdx.x < ma) {
-    double sum = 0.0;
-    for (int bl = 0; bl < (int)gridDim.x; ++bl) sum += partials[(size_t)bl * MAXB + threadIdx.x];
-    g[threadIdx.x] = sum;
+  // the blocks' sums, a warp per column (one thread per column took 608 loads
+  // and additions in a row)
+  for (int i = wi; i < ma; i += nw) {
+    const double sum = warp_sum_strided(partials + i, (int)gridDim.x, MAXB);
+    if (lane == 0) g[i] = sum;
   }
   if (threadIdx.x == 0) *counter = 0u;
 }
@@ -380,7 +380,6 @@ __global__ void __launch_bounds__(RED_THREADS, 4)
               const S* __restrict__ w, double* rr, double* partials, unsigned* counter) {
   using Rg = Ar<S>;
   using V = typename Rg::T;
-  __shared__ double sh[32];
   __shared__ V scc[MMAX];
   const int mm = m_dev ? min(max(*m_dev, 0), m) : m;
   if (threadIdx.x < MMAX) {
@@ -431,7 +430,7 @@ __global__ void __launch_bounds__(RED_THREADS, 4)
     if (rr) resid(s0, k, v);
   }
   if (!rr) return;
-  reduce_to<S>(v, rr, partials, counter, sh);
+  reduce_to<S>(v, rr, partials, counter);
 }
 
 // One classical Gram-Schmidt pass fused with the next pass's projections:
@@ -445,7 +444,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
                    double* partials, unsigned* counter) {
   using Rg = Ar<S>;
   using V = typename Rg::T;
-  __shared__ double sh[MMAX * 32];
+  __shared__ double sh[MMAX][RED_THREADS / 32], tot[MMAX];
   __shared__ V scc[MMAX];
   pdl_wait();
   const int mm = m_dev ? min(max(*m_dev, 0), m) : m;
@@ -471,16 +470,9 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
   }
 #pragma unroll
   for (int i = 0; i < MMAX; ++i) hacc[i] = Rg::dfin(hacc[i]);
-  double o1[MMAX];
-  block_sum_v<S, MMAX>(hacc, o1, sh);
-  if (publish_partials<MMAX>(o1, partials, counter)) {
-    double o[MMAX];
-    finish_sum<MMAX>(partials, counter, o, sh);
-    // the block sums are complete in thread 0 only
-    if (threadIdx.x == 0)
-      for (int q = 0; q < mm; ++q) h[q] = o[q];
-  }
   pdl_launch_dependents();
+  if (grid_sum_v<S>(hacc, sh, tot, partials, counter) && (int)threadIdx.x < mm)
+    h[threadIdx.x] = tot[threadIdx.x];
 }
 
 // Gram-Schmidt acceptance: if |r_src|^2 after orthogonalisation exceeds
@@ -718,10 +710,10 @@ static inline int vgrid(long long n) {
 cudaError_t launch_vdot(long long n, int vt, const void* a, const void* b, double* partials,
                         unsigned* counter, double* out, cudaStream_t s) {
   if (vt == V_DF2)
-    k_vdot<float2><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, (const float2*)a, (const float2*)b,
+    k_vdot<float2><<<vgrid(n), RED_THREADS, 0, s>>>(n, (const float2*)a, (const float2*)b,
                                                       partials, counter, out);
   else
-    k_vdot<double><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, (const double*)a, (const double*)b,
+    k_vdot<double><<<vgrid(n), RED_THREADS, 0, s>>>(n, (const double*)a, (const double*)b,
                                                       partials, counter, out);
   return cudaGetLastError();
 }
@@ -786,10 +778,13 @@ static void gram_t(long long n, const void* A, int na, const int* na_dev, const 
   });
   if (nb == 1 && nb_dev == nullptr && !sym) {
     const int wpc = na >= 8 ? 1 : 8 / na;   // warps per column
-    k_gram_col<S><<<RED_BLOCKS, 32 * na * wpc, 0, s>>>(n, (const S*)A, na, na_dev,
+    // (four to eight indices a lane at least)
+    const int gb = (int)std::min<long long>((n + 256LL * wpc - 1) / (256LL * wpc), RED_BLOCKS);
+    k_gram_col<S><<<gb, 32 * na * wpc, 0, s>>>(n, (const S*)A, na, na_dev,
                                                        (const S*)B, G, partials, counter);
   } else
-    k_gram<S><<<RED_BLOCKS, MD_CH, (size_t)2 * (na + nb) * MD_CH * sizeof(S), s>>>(
+    k_gram<S><<<(int)std::min<long long>((n + 2 * MD_CH - 1) / (2 * MD_CH), RED_BLOCKS), MD_CH,
+                (size_t)2 * (na + nb) * MD_CH * sizeof(S), s>>>(
         n, (const S*)A, na, na_dev, (const S*)B, nb, nb_dev, G, ldg, partials, counter, sym);
 }
 
@@ -822,16 +817,16 @@ static void combine_t(long long n, const void* A, int m, const int* m_dev, const
   const S* ww = (const S*)w;
   SY* yy = (SY*)y;
   if (m <= 4)
-    k_combine<S, SY, 4><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy, ww,
+    k_combine<S, SY, 4><<<vgrid(n), RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy, ww,
                                                            rr, partials, counter);
   else if (m <= 8)
-    k_combine<S, SY, 8><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy, ww,
+    k_combine<S, SY, 8><<<vgrid(n), RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy, ww,
                                                            rr, partials, counter);
   else if (m <= 12)
-    k_combine<S, SY, 12><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy,
+    k_combine<S, SY, 12><<<vgrid(n), RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy,
                                                             ww, rr, partials, counter);
   else
-    k_combine<S, SY, MAXB><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy,
+    k_combine<S, SY, MAXB><<<vgrid(n), RED_THREADS, 0, s>>>(n, a, m, m_dev, c, sign, beta, yy,
                                                               ww, rr, partials, counter);
 }
 
@@ -841,15 +836,15 @@ cudaError_t launch_combine_dots(long long n, int vt, const void* A, int m, const
   if (m > 12 || m < 0) return cudaErrorInvalidValue;
   if (vt == V_DF2) {
     if (m <= 4)
-      return launch_pdl(k_combine_dots<float2, 4>, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n,
+      return launch_pdl(k_combine_dots<float2, 4>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
                         (const float2*)A, m, m_dev, c, (float2*)y, h, partials, counter);
-    return launch_pdl(k_combine_dots<float2, 12>, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n,
+    return launch_pdl(k_combine_dots<float2, 12>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
                       (const float2*)A, m, m_dev, c, (float2*)y, h, partials, counter);
   }
   if (m <= 4)
-    return launch_pdl(k_combine_dots<double, 4>, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n,
+    return launch_pdl(k_combine_dots<double, 4>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
                       (const double*)A, m, m_dev, c, (double*)y, h, partials, counter);
-  return launch_pdl(k_combine_dots<double, 12>, dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s, n,
+  return launch_pdl(k_combine_dots<double, 12>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
                     (const double*)A, m, m_dev, c, (double*)y, h, partials, counter);
 }
 
