@@ -5,6 +5,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cstdlib>
 
 #include "dfmath.cuh"
 #include "kernels.h"
@@ -76,77 +77,189 @@ __global__ void __launch_bounds__(256)
     out[e] = 1.0 / acc;
 }
 
-// Double-float Walsh blocks of KE (hi and lo parts of each float64 entry)
+// 3D filter with offsets of at most R elements per axis (1 < rmin <= R + 1).
+// The weight depends on dx^2 + dy^2 + dz^2 alone, so a layer's values are first
+// summed over the offsets of equal dx^2 + dy^2 (s = 0, 1, 2 and, for R = 2, 4, 5,
+// 8), and each sum enters the 2R + 1 layers around it with one FMA: 15 (R = 1) or
+// at most 45 (R = 2) float64 instructions per element instead of two per
+// offset (27 to 93 offsets), on a pipe that does two per clock per SM.  A block
+// owns 32 x 4 columns of FLZ elements; their values with a halo (zero outside
+// the grid) are all requested at once and staged in shared memory, where the
+// factor invHs of the transpose is applied once, and a thread then runs up its
+// column.  Transpose at 192 x 96 x 96, offset list / this: rmin 1.5 131 / 62 us,
+// 2.0 184 / 74 us, 2.5 542 / 186 us; 64 x 32 x 32, 1.5: 10 / 8 us.  (One layer
+// staged at a time: 110 us at rmin 2.0, 24 us on small grids; 8 rows instead of
+// 4: 2 to 4 us more on small grids; weights of 0 tested at run time: float64
+// comparisons, as dear as the FMAs.)
+constexpr int FLX = 32, FLY = 4, FLZ = 4;
+
+template <int R>
+struct FilterW {
+  static constexpr int NS = R == 1 ? 3 : 6;   // classes of dx^2 + dy^2
+  double w[NS][R + 1];                        // weight of class s at |dz| = m
+};
+// dx^2 + dy^2 of class q
+__host__ __device__ constexpr int filter_class(int q) {
+  return q < 3 ? q : q == 3 ? 4 : q == 4 ? 5 : 8;
+}
+
+// D: the largest dx^2 + dy^2 + dz^2 inside the radius
+template <int R, int D>
+__global__ void __launch_bounds__(FLX * FLY)
+    k_filter3(GridP g, FilterW<R> fw, bool sens, const double* __restrict__ invHs,
+              const double* __restrict__ in, double* __restrict__ out) {
+  constexpr int NS = FilterW<R>::NS, SX = FLX + 2 * R, SY = FLY + 2 * R, SZ = FLZ + 2 * R;
+  __shared__ double t[SZ][SY][SX];
+  const int tid = threadIdx.x, tx = tid % FLX, ty = tid / FLX;
+  const int x0 = blockIdx.x * FLX, y0 = blockIdx.y * FLY, z0 = blockIdx.z * FLZ;
+  const long long plane = (long long)g.nx * g.ny;
+#pragma unroll 8
+  for (int q = tid; q < SX * SY * SZ; q += FLX * FLY) {
+    const int c = q % SX, r = q / SX % SY, l = q / (SX * SY);
+    const int jx = x0 - R + c, jy = y0 - R + r, jz = z0 - R + l;
+    const bool ok = jx >= 0 && jx < g.nx && jy >= 0 && jy < g.ny && jz >= 0 && jz < g.nz;
+    const long long j = ok ? jx + (long long)g.nx * jy + plane * jz : 0;
+    t[l][r][c] = ok ? (sens ? in[j] * invHs[j] : in[j]) : 0.0;
+  }
+  __syncthreads();
+  if (x0 + tx >= g.nx || y0 + ty >= g.ny) return;
+  double acc[2 * R + 1];   // acc[i]: the output of layer l - 2 R + i so far
+#pragma unroll
+  for (int i = 0; i < 2 * R + 1; ++i) acc[i] = 0.0;
+#pragma unroll
+  for (int l = 0; l < SZ; ++l) {
+    auto at = [&](int dx, int dy) { return t[l][ty + R + dy][tx + R + dx]; };
+    double v[NS];
+    v[0] = at(0, 0);
+    v[1] = (at(-1, 0) + at(1, 0)) + (at(0, -1) + at(0, 1));
+    if constexpr (D >= 2) v[2] = (at(-1, -1) + at(1, -1)) + (at(-1, 1) + at(1, 1));
+    if constexpr (R == 2) {
+      v[3] = (at(-2, 0) + at(2, 0)) + (at(0, -2) + at(0, 2));
+      if constexpr (D >= 5)
+        v[4] = ((at(-2, -1) + at(2, -1)) + (at(-2, 1) + at(2, 1))) +
+               ((at(-1, -2) + at(1, -2)) + (at(-1, 2) + at(1, 2)));
+      if constexpr (D >= 8) v[5] = (at(-2, -2) + at(2, -2)) + (at(-2, 2) + at(2, 2));
+    }
+#pragma unroll
+    for (int i = 0; i < 2 * R + 1; ++i) {
+      const int zo = l - 2 * R + i, m = i < R ? R - i : i - R;   // output layer, |dz|
+      if (zo < 0 || zo >= FLZ) continue;
+#pragma unroll
+      for (int q = 0; q < NS; ++q)
+        if (filter_class(q) + m * m <= D) acc[i] = fma(fw.w[q][m], v[q], acc[i]);
+    }
+    const int zo = l - 2 * R;
+    if (zo >= 0 && z0 + zo < g.nz) {
+      const long long e = x0 + tx + (long long)g.nx * (y0 + ty) + plane * (z0 + zo);
+      out[e] = sens ? acc[0] : acc[0] * invHs[e];
+    }
+#pragma unroll
+    for (int i = 0; i < 2 * R; ++i) acc[i] = acc[i + 1];
+    acc[2 * R] = 0.0;
+  }
+}
+
+template <int R, int D>
+static cudaError_t run_filter3(const GridP& g, const StencilP& st, bool sens, const double* invHs,
+                               const double* in, double* out, cudaStream_t s) {
+  FilterW<R> fw = {};
+  for (int q = 0; q < st.count; ++q) {
+    const int d2 = st.d[q][0] * st.d[q][0] + st.d[q][1] * st.d[q][1];
+    for (int c = 0; c < FilterW<R>::NS; ++c)
+      if (filter_class(c) == d2) fw.w[c][std::abs(st.d[q][2])] = st.w[q];
+  }
+  k_filter3<R, D><<<dim3((g.nx + FLX - 1) / FLX, (g.ny + FLY - 1) / FLY, (g.nz + FLZ - 1) / FLZ),
+                    FLX * FLY, 0, s>>>(g, fw, sens, invHs, in, out);
+  return cudaGetLastError();
+}
+
+// Double-float Walsh blocks of KE (hi and lo parts of each float64 entry), the
+// entries above the diagonal doubled: X^T B X = sum of the upper triangles
 struct WhtDf {
   float h[8][3][3], l[8][3][3];
 };
 
+__device__ __forceinline__ void wht4_dfl(dfl (&v)[4]) {
+  const dfl s0 = df_add(v[0], v[1]), d0 = df_add(v[0], df_neg(v[1]));
+  const dfl s1 = df_add(v[2], v[3]), d1 = df_add(v[2], df_neg(v[3]));
+  v[0] = df_add(s0, s1);
+  v[1] = df_add(d0, d1);
+  v[2] = df_add(s0, df_neg(s1));
+  v[3] = df_add(d0, df_neg(d1));
+}
+
 // 3D compliance and sensitivity of k_sensitivity3_wht in double-float
 // arithmetic (mixed path), for an integer penalisation exponent:
 // dc_e = pfac rho_e^ipen ce_e with pfac = -penal (E0 - Emin), ipen = penal - 1.
-__global__ void __launch_bounds__(RED_THREADS)
-    k_sensitivity3_df(GridP g, const uint8_t* __restrict__ mask, WhtDf kb,
+// A thread streams one element column in z: a face's twelve displacements are
+// loaded, split and xy-transformed once for the element below and the one
+// above (one element per thread read, split and transformed 24: 334 us at
+// 192 x 96 x 96), and the quadratic form takes the 33 non-zero entries of the
+// blocks' upper triangles instead of all 72.
+constexpr int SNX = 32, SNY = 4;
+__global__ void __launch_bounds__(SNX * SNY)
+    k_sensitivity3_df(GridP g, const uint8_t* __restrict__ mask, WhtDf kb, int zc,
                       const double* __restrict__ u, const double* __restrict__ E,
                       const double* __restrict__ rho, double pfac, int ipen,
                       double* __restrict__ dc, double* compliance, double* partials,
                       unsigned* counter) {
-  __shared__ double sh[32];
+  __shared__ double sh[1][SNX * SNY / 32], tot[1];
+  const int ex = blockIdx.x * SNX + threadIdx.x % SNX, ey = blockIdx.y * SNY + threadIdx.x / SNX;
+  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, g.nz);
+  const long long plane = (long long)g.nnx * g.nny;
   const dfl pf = split_d(pfac);
   dfl v[1] = {{0.f, 0.f}};
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < g.nel;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int ex = (int)(e % g.nx);
-    const long long rest = e / g.nx;
-    const int ey = (int)(rest % g.ny);
-    const int ez = (int)(rest / g.ny);
-    dfl X[3][8];
+  if (ex < g.nx && ey < g.ny) {
+    auto face = [&](int kz, dfl (&W)[3][4]) {
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const int i = ex + (a & 1), j = ey + ((a >> 1) & 1), k = ez + ((a >> 2) & 1);
-      const long long nd = i + (long long)g.nnx * (j + (long long)g.nny * k);
-      const unsigned m = mask[nd];
+      for (int q = 0; q < 4; ++q) {
+        const long long nd = ex + (q & 1) + (long long)g.nnx * (ey + (q >> 1)) + plane * kz;
+        const unsigned m = mask[nd];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          W[c][q] = ((m >> c) & 1u) ? dfl{0.f, 0.f} : split_d(u[3 * nd + c]);
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) wht4_dfl(W[c]);
+    };
+    dfl Wb[3][4], Wt[3][4];
+    face(z0, Wb);
+    for (int ez = z0; ez < z1; ++ez) {
+      const long long e = ex + (long long)g.nx * (ey + (long long)g.ny * ez);
+      const double re64 = rho[e], e64 = E[e];
+      face(ez + 1, Wt);
+      dfl X[3][8];
 #pragma unroll
       for (int c = 0; c < 3; ++c)
-        X[c][a] = ((m >> c) & 1u) ? dfl{0.f, 0.f} : split_d(u[3 * nd + c]);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          X[c][t] = df_add(Wb[c][t], Wt[c][t]);
+          X[c][t + 4] = df_add(Wb[c][t], df_neg(Wt[c][t]));
+          Wb[c][t] = Wt[c][t];
+        }
+      dfl ce = {0.f, 0.f};
+#pragma unroll
+      for (int tau = 0; tau < 8; ++tau)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          if (wht_zero(tau, c, c)) continue;   // (its row and column are zero too)
+          const dfl z = X[c][tau ^ (1 << c)];
+          dfl s = df_mul(dfl{kb.h[tau][c][c], kb.l[tau][c][c]}, z);
+#pragma unroll
+          for (int cp = c + 1; cp < 3; ++cp)
+            if (!wht_zero(tau, c, cp))
+              s = df_add(df_mul(dfl{kb.h[tau][c][cp], kb.l[tau][c][cp]}, X[cp][tau ^ (1 << cp)]),
+                         s);
+          ce = df_add(df_mul(z, s), ce);
+        }
+      const dfl re = split_d(re64);
+      dfl f = pf;
+      for (int q = 0; q < ipen; ++q) f = df_mul(f, re);
+      dc[e] = df_to_d(df_mul(f, ce));
+      v[0] = df_add(df_mul(split_d(e64), ce), v[0]);
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int h = 1; h < 8; h <<= 1)
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-          if (!(a & h)) {
-            const dfl p = X[c][a], q = X[c][a + h];
-            X[c][a] = df_add(p, q);
-            X[c][a + h] = df_add(p, df_neg(q));
-          }
-    dfl ce = {0.f, 0.f};
-#pragma unroll
-    for (int tau = 0; tau < 8; ++tau) {
-      dfl z[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) z[c] = X[c][tau ^ (1 << c)];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        dfl s = df_mul(dfl{kb.h[tau][c][0], kb.l[tau][c][0]}, z[0]);
-        s = df_add(df_mul(dfl{kb.h[tau][c][1], kb.l[tau][c][1]}, z[1]), s);
-        s = df_add(df_mul(dfl{kb.h[tau][c][2], kb.l[tau][c][2]}, z[2]), s);
-        ce = df_add(df_mul(z[c], s), ce);
-      }
-    }
-    const dfl re = split_d(rho[e]);
-    dfl f = pf;
-    for (int q = 0; q < ipen; ++q) f = df_mul(f, re);
-    dc[e] = df_to_d(df_mul(f, ce));
-    v[0] = df_add(df_mul(split_d(E[e]), ce), v[0]);
   }
-  double o1[1];
-  block_sum_df<1>(v, o1, sh);
-  if (publish_partials<1>(o1, partials, counter)) {
-    double o[1];
-    finish_sum<1>(partials, counter, o, sh);
-    if (threadIdx.x == 0) *compliance = o[0];
-  }
+  if (grid_sum_df(v, sh, tot, partials, counter) && threadIdx.x == 0) *compliance = tot[0];
 }
 
 // ce_e = u_e^T KE u_e; dc_e = -penal (E0-Emin) rho_e^(penal-1) ce_e;
@@ -532,6 +645,18 @@ cudaError_t launch_filter(int dim, const GridP& g, const StencilP& st, int mode,
                           const double* Hs, const double* in, double* out, cudaStream_t s) {
   if (dim == 2)
     k_filter<2><<<nblocks(g.nel, 256), 256, 0, s>>>(g, st, mode, Hs, in, out);
+  else if (mode != 2 && st.reach >= 1 && st.reach <= 2) {
+    const bool sens = mode == 1;
+    switch (st.d2max) {
+      case 1: return run_filter3<1, 1>(g, st, sens, Hs, in, out, s);
+      case 2: return run_filter3<1, 2>(g, st, sens, Hs, in, out, s);
+      case 3: return run_filter3<1, 3>(g, st, sens, Hs, in, out, s);
+      case 4: return run_filter3<2, 4>(g, st, sens, Hs, in, out, s);
+      case 5: return run_filter3<2, 5>(g, st, sens, Hs, in, out, s);
+      case 6: return run_filter3<2, 6>(g, st, sens, Hs, in, out, s);
+      default: return run_filter3<2, 8>(g, st, sens, Hs, in, out, s);
+    }
+  }
   else
     k_filter<3><<<nblocks(g.nel, 256), 256, 0, s>>>(g, st, mode, Hs, in, out);
   return cudaGetLastError();
@@ -549,13 +674,18 @@ cudaError_t launch_sensitivity_df(const GridP& g, const uint8_t* mask, const dou
   if (!wht || !sensitivity_df_ok(3, penal)) return cudaErrorInvalidValue;
   WhtDf kb;
   for (int q = 0; q < 72; ++q) {
-    const float h = (float)wht[q];
+    const double w = (q % 3 > q / 3 % 3 ? 2.0 : 1.0) * wht[q];
+    const float h = (float)w;
     (&kb.h[0][0][0])[q] = h;
-    (&kb.l[0][0][0])[q] = (float)(wht[q] - (double)h);
+    (&kb.l[0][0][0])[q] = (float)(w - (double)h);
   }
-  k_sensitivity3_df<<<RED_BLOCKS, RED_THREADS, 0, s>>>(g, mask, kb, u, E, rho,
-                                                       -penal * (E0 - Emin), (int)penal - 1, dc,
-                                                       compliance, partials, counter);
+  const int gx = (g.nx + SNX - 1) / SNX, gy = (g.ny + SNY - 1) / SNY;
+  // z-chunk: its first face is loaded and transformed again
+  int zc = 16;
+  while (zc > 1 && (long long)gx * gy * ((g.nz + zc - 1) / zc) < 4 * 152) zc /= 2;
+  k_sensitivity3_df<<<dim3(gx, gy, (g.nz + zc - 1) / zc), SNX * SNY, 0, s>>>(
+      g, mask, kb, zc, u, E, rho, -penal * (E0 - Emin), (int)penal - 1, dc, compliance, partials,
+      counter);
   return cudaGetLastError();
 }
 

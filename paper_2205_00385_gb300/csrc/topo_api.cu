@@ -222,7 +222,7 @@ static void grandchild_galerkin(const double* Qc, double* R) {
 
 static bool make_stencil(int dim, double rmin, StencilP* st) {
   const int R = (int)ceil(rmin);
-  st->count = 0;
+  st->count = st->reach = st->d2max = 0;
   for (int dz = (dim == 3 ? -R : 0); dz <= (dim == 3 ? R : 0); ++dz)
     for (int dy = -R; dy <= R; ++dy)
       for (int dx = -R; dx <= R; ++dx) {
@@ -233,6 +233,8 @@ static bool make_stencil(int dim, double rmin, StencilP* st) {
         st->d[st->count][1] = dy;
         st->d[st->count][2] = dz;
         st->w[st->count] = w;
+        st->reach = std::max({st->reach, abs(dx), abs(dy), abs(dz)});
+        st->d2max = std::max(st->d2max, dx * dx + dy * dy + dz * dz);
         st->count++;
       }
   return true;

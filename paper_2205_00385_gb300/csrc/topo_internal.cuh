@@ -103,7 +103,7 @@ __device__ __forceinline__ void fwht8(TC (&v)[8]) {
 }
 
 struct StencilP {
-  int count;
+  int count, reach, d2max;   // offsets, the largest along an axis, the largest squared length
   int d[MAX_STENCIL][3];
   double w[MAX_STENCIL];
 };
@@ -281,6 +281,8 @@ __device__ __forceinline__ bool grid_sum(double (&sh)[NV][NW], double (&out)[NV]
   static_assert((NW & (NW - 1)) == 0 && NW <= 32, "a power of two of warps");
   __shared__ bool s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned nblk = gridDim.x * gridDim.y * gridDim.z;
+  const size_t blk = blockIdx.x + (size_t)gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
   __syncthreads();
 #pragma unroll
   for (int q0 = 0; q0 < NV; q0 += NW) {
@@ -289,12 +291,12 @@ __device__ __forceinline__ bool grid_sum(double (&sh)[NV][NW], double (&out)[NV]
 #pragma unroll
     for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
     if (lane == 0 && q < NV) {
-      partials[(size_t)blockIdx.x * NV + q] = t;
+      partials[blk * NV + q] = t;
       __threadfence();   // (the writing threads only: a fence waits for all stores of its thread)
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == nblk - 1;
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
@@ -302,7 +304,7 @@ __device__ __forceinline__ bool grid_sum(double (&sh)[NV][NW], double (&out)[NV]
   for (int q0 = 0; q0 < NV; q0 += NW) {
     const int q = q0 + warp;
     if (q >= NV) break;
-    const double t = warp_sum_strided(partials + q, (int)gridDim.x, NV);
+    const double t = warp_sum_strided(partials + q, (int)nblk, NV);
     if (lane == 0) out[q] = t;
   }
   if (threadIdx.x == 0) *counter = 0u;
