@@ -307,15 +307,15 @@ cudaError_t launch_oc_step(long long nel, const double* rho, const double* a,
 // lambda search of the OC update: the candidate factors
 // a = rho max(0, -dc/dv)^eta (float64 copy a64 for the final update; eta
 // 1/2 for compliance), the move limits and dv as double-float pairs and the
-// first bracket; one sweep narrows the bracket in double-float (a no-op once
-// it is within 1e-13); rho_new = clamp(a lambda^-eta)
+// first bracket; the search narrows the bracket to 1e-13 in double-float;
+// rho_new = clamp(a lambda^-eta)
 cudaError_t launch_oc_prep_d(long long nel, const double* rho, const double* dc,
                              const double* dv, double move, double target, double* a64, void* a2,
                              void* lo2, void* hi2, void* dv2, double* scal, double* partials,
                              unsigned* counter, cudaStream_t s, double eta = 0.5);
-cudaError_t launch_oc_sweep(long long nel, const void* a2, const void* lo2, const void* hi2,
-                            const void* dv2, double target, double* scal, double* partials,
-                            unsigned* counter, cudaStream_t s, double eta = 0.5);
+cudaError_t launch_oc_search(long long nel, const void* a2, const void* lo2, const void* hi2,
+                             const void* dv2, double target, double* scal, double* partials,
+                             unsigned* counter, cudaStream_t s, double eta = 0.5);
 cudaError_t launch_oc_final(long long nel, double* rho, const double* a, double move,
                             double* scal, double* change_dev, double* partials,
                             unsigned* counter, cudaStream_t s, double eta = 0.5);

@@ -194,10 +194,10 @@ __device__ __forceinline__ void wht4_dfl(dfl (&v)[4]) {
 // A thread streams one element column in z: a face's twelve displacements are
 // loaded, split and xy-transformed once for the element below and the one
 // above (one element per thread read, split and transformed 24: 334 us at
-// 192 x 96 x 96), and the quadratic form takes the 33 non-zero entries of the
+// 192 x 96 x 96, now 158), and the quadratic form takes the 33 non-zero entries of the
 // blocks' upper triangles instead of all 72.
 constexpr int SNX = 32, SNY = 4;
-__global__ void __launch_bounds__(SNX * SNY)
+__global__ void __launch_bounds__(SNX * SNY, 6)
     k_sensitivity3_df(GridP g, const uint8_t* __restrict__ mask, WhtDf kb, int zc,
                       const double* __restrict__ u, const double* __restrict__ E,
                       const double* __restrict__ rho, double pfac, int ipen,
@@ -429,9 +429,12 @@ __global__ void __launch_bounds__(RED_THREADS)
 //                    1/32 of that, and the bracket's thirds, which bound the
 //                    sweeps when the secant point misses
 // Six or seven sweeps reach the relative bracket of 1e-13 (equal sections of
-// the bracket took 17 to 23); a sweep after that is a no-op.  A sweep reads
-// 32 bytes per element (57 MB at 192 x 96 x 96, which stays in L2).
-constexpr int OC_NP = 7, OC_T = 512, OC_BLOCKS = 304;
+// the bracket took 17 to 23); a sweep after that is a no-op, and one block
+// goes on where OC_SWEEPS were not enough, so that nothing waits for the host
+// and a captured update needs no more launches.  A sweep reads 32 bytes per
+// element (57 MB at 192 x 96 x 96, which stays in L2): 24 us there, of which the
+// arithmetic of the seven points is 8.
+constexpr int OC_NP = 7, OC_T = 512, OC_BLOCKS = 304, OC_SWEEPS = 9;
 constexpr double OC_LAM_MAX = 1e9;
 static_assert(OC_NP <= S_OC_NPT && OC_NP <= OC_T / 32, "one warp per point");
 
@@ -453,9 +456,11 @@ __device__ __forceinline__ bool oc_done(double l1, double l2) {
 }
 
 // Writes the bracket and its next points; called by one whole warp.
+// v1, v2 and s1, s2: the volumes and factors lambda^-eta at the bracket's ends
+// (of the lower end unknown, and not used, while it is 0).
 __device__ __forceinline__ void oc_next_points(double l1, double l2, double v1, double v2,
-                                               double target, double eta, double l0,
-                                               double* scal) {
+                                               double s1, double s2, double target, double eta,
+                                               double l0, volatile double* scal) {
   const int j = threadIdx.x & 31;
   double lam;
   if (l0 > 0.0) {
@@ -466,11 +471,10 @@ __device__ __forceinline__ void oc_next_points(double l1, double l2, double v1, 
     const double q = sqrt(sqrt(sqrt(l2 / l1)));
     lam = l1;
     for (int i = 0; i <= j && i < OC_NP; ++i) lam *= q;
-  } else if (!(v1 > v2)) {   // a volume not known (or no slope): equal sections
+  } else if (!(v1 > v2)) {   // no slope: equal sections
     lam = l1 + (j + 1) * ((l2 - l1) / (OC_NP + 1));
   } else {
-    const double sa = oc_lam_factor(l2, eta), sb = oc_lam_factor(l1, eta);
-    const double mid = oc_lam_of(sa + (target - v2) * ((sb - sa) / (v1 - v2)), eta);
+    const double mid = oc_lam_of(s2 + (target - v2) * ((s1 - s2) / (v1 - v2)), eta);
     const double w = (l2 - l1) / l2, d = mid * fmax(0.5 * w * w, 6.4e-13);
     lam = j == 0 ? mid - d
         : j == 1 ? mid - d / 32
@@ -496,6 +500,8 @@ __device__ __forceinline__ void oc_next_points(double l1, double l2, double v1, 
     scal[S_OC_L2] = l2;
     scal[S_OC_V1] = v1;
     scal[S_OC_V2] = v2;
+    scal[S_OC_S1] = s1;
+    scal[S_OC_S2] = s2;
   }
 }
 
@@ -538,53 +544,65 @@ __global__ void __launch_bounds__(OC_T)
   const double l0 = oc_lam_of(target / tot[0], eta);
   const double l1 = tot[1] > target && tot[2] > target ? OC_LAM_MAX : 0.0;
   const double l2 = tot[1] > target ? OC_LAM_MAX : 0.0;
-  oc_next_points(l1, l2, tot[1], tot[2], target, eta,
+  const double st = oc_lam_factor(OC_LAM_MAX, eta);
+  oc_next_points(l1, l2, tot[1], tot[2], st, st, target, eta,
                  l0 > 1e-60 && l0 < OC_LAM_MAX ? l0 : 0.0, scal);
 }
 
+// One sweep by the whole grid (LOOP: by one block, until the bracket is done;
+// a sweep at least thirds a bracket that does not start at 0 and takes one that
+// does down by 8^7, so the limit is not met).
+template <bool LOOP>
 __global__ void __launch_bounds__(OC_T, 2)
     k_oc_sweep(long long nel, const float4* __restrict__ a, const float4* __restrict__ lo,
                const float4* __restrict__ hi, const float4* __restrict__ dvd, double target,
-               double* scal, double* partials, unsigned* counter, double eta) {
+               volatile double* scal, double* partials, unsigned* counter, double eta) {
   __shared__ double sh[OC_NP][OC_T / 32], tot[OC_NP];
   pdl_wait();
-  const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
-  if (oc_done(l1, l2)) return;
-  dfl sv[OC_NP], v[OC_NP];
-#pragma unroll
-  for (int j = 0; j < OC_NP; ++j) {
-    sv[j] = split_d(scal[S_OC_SP + j]);
-    v[j] = {0.f, 0.f};
-  }
-  auto element = [&](dfl av, dfl lv, dfl hv, dfl dd) {
+  for (int it = 0; it < (LOOP ? 160 : 1); ++it) {
+    const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
+    if (oc_done(l1, l2)) return;
+    dfl sv[OC_NP], v[OC_NP];
 #pragma unroll
     for (int j = 0; j < OC_NP; ++j) {
-      dfl x = df_mul(av, sv[j]);
-      x = df_gt(x, hv) ? hv : (df_gt(lv, x) ? lv : x);
-      df_dot_acc(v[j], dd, x);
+      sv[j] = split_d(scal[S_OC_SP + j]);
+      v[j] = {0.f, 0.f};
     }
-  };
-  // two elements per 16-byte load (nel is even: every grid coarsens once)
-  for (long long q = (long long)blockIdx.x * OC_T + threadIdx.x; 2 * q < nel;
-       q += (long long)gridDim.x * OC_T) {
-    const float4 a4 = a[q], l4 = lo[q], h4 = hi[q], d4 = dvd[q];
-    element({a4.x, a4.y}, {l4.x, l4.y}, {h4.x, h4.y}, {d4.x, d4.y});
-    element({a4.z, a4.w}, {l4.z, l4.w}, {h4.z, h4.w}, {d4.z, d4.w});
-  }
+    auto element = [&](dfl av, dfl lv, dfl hv, dfl dd) {
 #pragma unroll
-  for (int j = 0; j < OC_NP; ++j) v[j] = df_norm(v[j]);
-  pdl_launch_dependents();
-  if (!grid_sum_df(v, sh, tot, partials, counter) || threadIdx.x >= 32) return;
-  // the volume decreases with lambda: keep the last point above target and
-  // the first at or below it
-  int k = 0;
-  while (k < OC_NP && tot[k] > target) ++k;
-  const double n1 = k > 0 ? scal[S_OC_PT + k - 1] : l1;
-  const double w1 = k > 0 ? tot[k - 1] : scal[S_OC_V1];
-  const double n2 = k < OC_NP ? scal[S_OC_PT + k] : l2;
-  const double w2 = k < OC_NP ? tot[k] : scal[S_OC_V2];
-  __syncwarp();
-  oc_next_points(n1, n2, w1, w2, target, eta, 0.0, scal);
+      for (int j = 0; j < OC_NP; ++j) {
+        dfl x = df_mul(av, sv[j]);
+        x = df_gt(x, hv) ? hv : (df_gt(lv, x) ? lv : x);
+        df_dot_acc(v[j], dd, x);
+      }
+    };
+    // two elements per 16-byte load (nel is even: every grid coarsens once)
+    for (long long q = (long long)blockIdx.x * OC_T + threadIdx.x; 2 * q < nel;
+         q += (long long)gridDim.x * OC_T) {
+      const float4 a4 = a[q], l4 = lo[q], h4 = hi[q], d4 = dvd[q];
+      element({a4.x, a4.y}, {l4.x, l4.y}, {h4.x, h4.y}, {d4.x, d4.y});
+      element({a4.z, a4.w}, {l4.z, l4.w}, {h4.z, h4.w}, {d4.z, d4.w});
+    }
+#pragma unroll
+    for (int j = 0; j < OC_NP; ++j) v[j] = df_norm(v[j]);
+    if (!LOOP) pdl_launch_dependents();
+    if (!grid_sum_df(v, sh, tot, partials, counter)) return;
+    if (threadIdx.x < 32) {
+      // the volume decreases with lambda: keep the last point above target
+      // and the first at or below it
+      int k = 0;
+      while (k < OC_NP && tot[k] > target) ++k;
+      const double n1 = k > 0 ? scal[S_OC_PT + k - 1] : l1;
+      const double w1 = k > 0 ? tot[k - 1] : scal[S_OC_V1];
+      const double f1 = scal[k > 0 ? S_OC_SP + k - 1 : S_OC_S1];
+      const double n2 = k < OC_NP ? scal[S_OC_PT + k] : l2;
+      const double w2 = k < OC_NP ? tot[k] : scal[S_OC_V2];
+      const double f2 = scal[k < OC_NP ? S_OC_SP + k : S_OC_S2];
+      __syncwarp();
+      oc_next_points(n1, n2, w1, w2, f1, f2, target, eta, 0.0, scal);
+    }
+    if (LOOP) __syncthreads();
+  }
 }
 
 // rho <- clamp(a lambda^-eta) and max |rho_new - rho|.  The limits are
@@ -680,9 +698,10 @@ cudaError_t launch_sensitivity_df(const GridP& g, const uint8_t* mask, const dou
     (&kb.l[0][0][0])[q] = (float)(w - (double)h);
   }
   const int gx = (g.nx + SNX - 1) / SNX, gy = (g.ny + SNY - 1) / SNY;
-  // z-chunk: its first face is loaded and transformed again
+  // z-chunk: its first face is loaded and transformed again, so as long as the
+  // blocks still fill the SMs (six resident on each)
   int zc = 16;
-  while (zc > 1 && (long long)gx * gy * ((g.nz + zc - 1) / zc) < 4 * 152) zc /= 2;
+  while (zc > 1 && (long long)gx * gy * ((g.nz + zc - 1) / zc) < 6 * 152) zc /= 2;
   k_sensitivity3_df<<<dim3(gx, gy, (g.nz + zc - 1) / zc), SNX * SNY, 0, s>>>(
       g, mask, kb, zc, u, E, rho, -penal * (E0 - Emin), (int)penal - 1, dc, compliance, partials,
       counter);
@@ -754,12 +773,18 @@ cudaError_t launch_oc_prep_d(long long nel, const double* rho, const double* dc,
   return cudaGetLastError();
 }
 
-cudaError_t launch_oc_sweep(long long nel, const void* a2, const void* lo2, const void* hi2,
-                            const void* dv2, double target, double* scal, double* partials,
-                            unsigned* counter, cudaStream_t s, double eta) {
-  return launch_pdl(k_oc_sweep, dim3(oc_blocks(nel)), dim3(OC_T), 0, s, nel, (const float4*)a2,
-                    (const float4*)lo2, (const float4*)hi2, (const float4*)dv2, target, scal,
-                    partials, counter, eta);
+cudaError_t launch_oc_search(long long nel, const void* a2, const void* lo2, const void* hi2,
+                             const void* dv2, double target, double* scal, double* partials,
+                             unsigned* counter, cudaStream_t s, double eta) {
+  auto sweep = [&](auto kern, int blocks) {
+    return launch_pdl(kern, dim3(blocks), dim3(OC_T), 0, s, nel, (const float4*)a2,
+                      (const float4*)lo2, (const float4*)hi2, (const float4*)dv2, target, scal,
+                      partials, counter, eta);
+  };
+  cudaError_t e = cudaSuccess;
+  for (int q = 0; q < OC_SWEEPS && e == cudaSuccess; ++q)
+    e = sweep(k_oc_sweep<false>, oc_blocks(nel));
+  return e == cudaSuccess ? sweep(k_oc_sweep<true>, 1) : e;
 }
 
 cudaError_t launch_oc_final(long long nel, double* rho, const double* a, double move,

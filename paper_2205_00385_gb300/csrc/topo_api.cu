@@ -1783,34 +1783,19 @@ to_status to_filter(to_ctx* c, int32_t mode, const double* in, double* out) {
 
 }  // extern "C"
 
-static to_status oc_prep(to_ctx* c, double target, double move, const double* dc_f,
-                         const double* dv_f, const double* rho) {
-  LAUNCH(c, launch_oc_prep_d(c->nel, rho, dc_f, dv_f, move, target, c->oc_a, c->oc_a2, c->oc_lo,
-                             c->oc_hi, c->oc_dv2, c->scal, c->partials, c->counters + C_OC,
-                             c->stream, c->oc_eta), "oc prep");
-  return TO_OK;
-}
-
-static to_status oc_sweeps(to_ctx* c, double target, int count) {
-  for (int q = 0; q < count; ++q)
-    LAUNCH(c, launch_oc_sweep(c->nel, c->oc_a2, c->oc_lo, c->oc_hi, c->oc_dv2, target, c->scal,
-                              c->partials, c->counters + C_OC, c->stream, c->oc_eta), "oc sweep");
-  return TO_OK;
-}
-
-// The OC update with a fixed number of sweeps of the multiplier search and
-// no host read, so that it can be captured into a graph: a sweep is a no-op
-// once the bracket is within 1e-13.  Every sweep of a narrow bracket at least
-// thirds it (28 to 1e-13); 8 more cover the way from [0, 1e9] to a narrow
-// one, so the result equals to_oc_update's.
+// The OC update; no host read, so that it can be captured into a graph.
 to_status oc_update_enqueue(to_ctx* c, double volfrac, double move, const double* dc_f,
                             const double* dv_f, double* rho, double* change_dev) {
-  const double target = volfrac * (double)c->nel;
-  to_status st;
-  if ((st = oc_prep(c, target, move, dc_f, dv_f, rho)) != TO_OK) return st;
-  if ((st = oc_sweeps(c, target, 36)) != TO_OK) return st;
-  LAUNCH(c, launch_oc_final(c->nel, rho, c->oc_a, move, c->scal, change_dev, c->partials,
-                            c->counters + C_MAX, c->stream, c->oc_eta), "oc final");
+  cudaStream_t s = c->stream;
+  const long long nel = c->nel;
+  const double target = volfrac * (double)nel;
+  LAUNCH(c, launch_oc_prep_d(nel, rho, dc_f, dv_f, move, target, c->oc_a, c->oc_a2, c->oc_lo,
+                             c->oc_hi, c->oc_dv2, c->scal, c->partials, c->counters + C_OC, s,
+                             c->oc_eta), "oc prep");
+  LAUNCH(c, launch_oc_search(nel, c->oc_a2, c->oc_lo, c->oc_hi, c->oc_dv2, target, c->scal,
+                             c->partials, c->counters + C_OC, s, c->oc_eta), "oc search");
+  LAUNCH(c, launch_oc_final(nel, rho, c->oc_a, move, c->scal, change_dev, c->partials,
+                            c->counters + C_MAX, s, c->oc_eta), "oc final");
   return TO_OK;
 }
 
@@ -1821,22 +1806,7 @@ to_status to_oc_update(to_ctx* c, double volfrac, double move, const double* dc_
   if (!c || !dc_f || !dv_f || !rho) return fail(c, TO_E_INVALID, "NULL argument");
   if (!(volfrac > 0.0 && volfrac <= 1.0) || !(move > 0.0 && move <= 1.0))
     return fail(c, TO_E_INVALID, "bad volfrac/move");
-  cudaStream_t s = c->stream;
-  const double target = volfrac * (double)c->nel;
-  to_status st;
-  if ((st = oc_prep(c, target, move, dc_f, dv_f, rho)) != TO_OK) return st;
-  // six or seven sweeps reach the final bracket, so eight are queued before
-  // the host looks, then eight more at a time
-  for (int chunk = 0; chunk < 16; ++chunk) {
-    if ((st = oc_sweeps(c, target, 8)) != TO_OK) return st;
-    double lr[2];
-    CUDA_TRY(c, cudaMemcpyAsync(lr, c->scal + S_OC_L1, 16, cudaMemcpyDeviceToHost, s), "read");
-    CUDA_TRY(c, cudaStreamSynchronize(s), "sync");
-    if (!((lr[1] - lr[0]) > 1e-13 * (lr[0] + lr[1]))) break;
-  }
-  LAUNCH(c, launch_oc_final(c->nel, rho, c->oc_a, move, c->scal, change_dev, c->partials,
-                            c->counters + C_MAX, s, c->oc_eta), "oc final");
-  return TO_OK;
+  return oc_update_enqueue(c, volfrac, move, dc_f, dv_f, rho, change_dev);
 }
 
 to_status to_profile_enable(to_ctx* c, int32_t kinds) {

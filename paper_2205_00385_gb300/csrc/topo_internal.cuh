@@ -113,9 +113,9 @@ enum Slot {
   S_RR = 0, S_PQ = 1, S_RZ0 = 2, S_RZ1 = 3, S_NRM = 4, S_TMP = 5, S_COMPL = 6,
   S_OC_L1 = 7, S_OC_L2 = 8, S_OC_VOL = 9, S_OC_DONE = 10, S_CHANGE = 11, S_EPS = 12,
   S_NRM0 = 13, S_NRM1 = 14, S_FNORM2 = 15, S_FLAG = 16,
-  // OC search: volumes at the bracket's ends, the sweep's multipliers and
-  // their factors lambda^-eta
-  S_OC_V1 = 17, S_OC_V2 = 18, S_OC_NPT = 8, S_OC_PT = 24, S_OC_SP = S_OC_PT + S_OC_NPT,
+  // OC search: volumes and factors lambda^-eta at the bracket's ends, the
+  // sweep's multipliers and their factors
+  S_OC_V1 = 17, S_OC_V2 = 18, S_OC_S1 = 19, S_OC_S2 = 20, S_OC_NPT = 8, S_OC_PT = 24, S_OC_SP = S_OC_PT + S_OC_NPT,
   S_NSLOTS = 64
 };
 
@@ -440,8 +440,7 @@ struct to_ctx {
   std::vector<double> ev_bytes;
 };
 
-// (topo_api.cu) the OC update with a fixed number of lambda sections and no
-// host read, capturable into a graph; same result as to_oc_update
+// (topo_api.cu) the OC update, capturable into a graph
 to_status oc_update_enqueue(to_ctx* c, double volfrac, double move, const double* dc_f,
                             const double* dv_f, double* rho, double* change_dev);
 // (batch.cu) drops the cached batch graphs that reference c
