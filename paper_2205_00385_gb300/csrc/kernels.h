@@ -134,16 +134,22 @@ cudaError_t launch_diag(int dim, const GridP& g, const uint8_t* mask, int tc, bo
 // b_c = Pm^T r_f; when zc is not null also the coarse level's smoothing from
 // a zero guess, zc = omega * dinvc * b_c.  clean: r_f is zero on every fixed
 // DOF (the fine masks are then not read; same result)
-cudaError_t launch_restrict(int dim, int t, const GridP& gf, const uint8_t* maskf,
-                            const GridP& gc, const uint8_t* maskc, const void* rf, void* bc,
-                            const void* dinvc, double omega, void* zc, bool clean,
+cudaError_t launch_restrict(int dim, int t, const GridP& gf, const GridP& gc, const uint8_t* mc,
+                            const void* rf, void* bc, const void* dinvc, double omega, void* zc,
                             cudaStream_t s);
 cudaError_t launch_prolong_add(int dim, int t, const GridP& gf, const uint8_t* maskf,
                                const GridP& gc, const void* zc, void* zf, cudaStream_t s);
-// z = omega * dinv * b (smoothing from a zero initial guess); if bout != 0 the
-// input (of type tin) is also converted into bout (type t).
+// z = omega * dinv * b (smoothing from a zero initial guess); the input (of
+// type tin) is also converted into bout (type t).
+// with a node mask the input is taken as zero on the fixed DOFs
 cudaError_t launch_presmooth(int t, int tin, long long n, const void* bin, void* bout,
-                             const void* dinv, double omega, void* z, cudaStream_t s);
+                             const void* dinv, double omega, void* z, cudaStream_t s, int dim = 0,
+                             const uint8_t* mask = nullptr);
+// float64 result of a V-cycle on an input r that may be nonzero on fixed DOFs:
+// out = zin (type t; null: out holds it already) on free DOFs, the operator
+// being the identity on fixed ones
+cudaError_t launch_vcycle_out(int dim, int t, long long n, const void* zin, const double* r,
+                              double omega, const uint8_t* mask, double* out, cudaStream_t s);
 cudaError_t launch_galerkin_fine(int dim, int t, const GridP& gc, const GridP& gf,
                                  const void* coef, const void* Qc, void* Kc, cudaStream_t s);
 cudaError_t launch_galerkin_coarse(int dim, int t, const GridP& gc, const GridP& gf,

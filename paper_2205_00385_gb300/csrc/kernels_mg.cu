@@ -27,14 +27,14 @@ namespace topo {
 // ---------------------------------------------------------------------------
 constexpr int TVAL = 256;
 
-// CLEAN: r_f is +-0 on every fixed DOF, so the fine masks are not loaded: a
-// fixed term then adds w * (+-0) where restrict_finish adds +0, and a
-// running sum that starts at +0 is never -0, so the bits are the same.
-template <int DIM, typename T, bool CLEAN>
+// r_f is +-0 on every fixed DOF (the cycle's input is cleared there), so the
+// fine masks are not loaded: a fixed term then adds w * (+-0) where
+// restrict_finish adds +0, and a running sum that starts at +0 is never -0,
+// so the bits are the same.
+template <int DIM, typename T>
 __global__ void __launch_bounds__(TVAL)
-    k_restrict(GridP gf, const uint8_t* __restrict__ maskf, GridP gc,
-               const uint8_t* __restrict__ maskc, const T* __restrict__ rf, T* __restrict__ bc,
-               const T* __restrict__ dinvc, T omega, T* __restrict__ zc) {
+    k_restrict(GridP gf, GridP gc, const uint8_t* __restrict__ maskc, const T* __restrict__ rf,
+               T* __restrict__ bc, const T* __restrict__ dinvc, T omega, T* __restrict__ zc) {
   constexpr int NZ = DIM == 3 ? 3 : 1;
   const int rowv = DIM * gc.nnx;
   const int pv = blockIdx.x * TVAL + threadIdx.x;
@@ -43,7 +43,6 @@ __global__ void __launch_bounds__(TVAL)
   if (pv >= rowv * gc.nny) return;
   const int J = pv / rowv, v = pv - J * rowv;
   const int I = v / DIM, c = v - I * DIM;
-  unsigned m[NZ][3][3];
   T x[NZ][3][3];
 #pragma unroll
   for (int a = 0; a < NZ; ++a)
@@ -54,9 +53,7 @@ __global__ void __launch_bounds__(TVAL)
         const int i = min(max(2 * I + q - 1, 0), gf.nnx - 1);
         const int j = min(max(2 * J + b - 1, 0), gf.nny - 1);
         const int k = DIM == 3 ? min(max(2 * K + a - 1, 0), gf.nnz - 1) : 0;
-        const long long fn = i + (long long)gf.nnx * (j + (long long)gf.nny * k);
-        m[a][b][q] = CLEAN ? 0u : (unsigned)maskf[fn];
-        x[a][b][q] = rf[DIM * fn + c];
+        x[a][b][q] = rf[DIM * (i + (long long)gf.nnx * (j + (long long)gf.nny * k)) + c];
       }
   T acc = T(0);
 #pragma unroll
@@ -70,8 +67,7 @@ __global__ void __launch_bounds__(TVAL)
         bool in = i >= 0 && i < gf.nnx && j >= 0 && j < gf.nny;
         if (DIM == 3) in = in && k >= 0 && k < gf.nnz;
         const T w = T((dx ? 0.5 : 1.0) * (dy ? 0.5 : 1.0) * (dz ? 0.5 : 1.0));
-        const unsigned mm = in ? m[a][b][q] : 7u;
-        acc = add_rn(acc, ((mm >> c) & 1u) ? T(0) : mul_rn(w, x[a][b][q]));
+        acc = add_rn(acc, in ? mul_rn(w, x[a][b][q]) : T(0));
       }
   const long long node = I + (long long)gc.nnx * (J + (long long)gc.nny * K);
   const long long d = DIM * node + c;
@@ -103,24 +99,83 @@ __global__ void __launch_bounds__(TBX * TBY, transfer_min_blocks<T>())
   pdl_launch_dependents();
 }
 
-template <typename T, typename TIN>
-__global__ void __launch_bounds__(256)
+// Element-wise passes: EW_U values per thread, a block's width apart, all
+// requested before any is used (one per thread left 24 and 16 us of a V-cycle
+// at 192 x 96 x 96 to these two passes).
+constexpr int EW_T = 256, EW_U = 4;
+
+// bout = bin and z = omega D^-1 bin (smoothing from a zero guess); with a node
+// mask (DIM > 0) the input is taken as zero on the fixed DOFs.
+template <int DIM, typename T, typename TIN>
+__global__ void __launch_bounds__(EW_T)
     k_presmooth(long long n, const TIN* __restrict__ bin, T* __restrict__ bout,
-                const T* __restrict__ dinv, T omega, T* __restrict__ z) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+                const T* __restrict__ dinv, T omega, T* __restrict__ z,
+                const uint8_t* __restrict__ mask) {
+  const long long q0 = (long long)blockIdx.x * EW_T * EW_U + threadIdx.x;
   pdl_wait();
-  if (q >= n) return;
-  const T bv = cvt<T>(bin[q]);
-  if (bout) bout[q] = bv;
-  z[q] = omega * dinv[q] * bv;
+  TIN bv[EW_U];
+  T dv[EW_U];
+  bool fx[EW_U];
+#pragma unroll
+  for (int u = 0; u < EW_U; ++u) {
+    const long long q = q0 + u * EW_T;
+    if (q >= n) continue;
+    bv[u] = bin[q];
+    dv[u] = dinv[q];
+    fx[u] = DIM > 0 && ((mask[q / (DIM > 0 ? DIM : 1)] >> (int)(q % (DIM > 0 ? DIM : 1))) & 1u);
+  }
+#pragma unroll
+  for (int u = 0; u < EW_U; ++u) {
+    const long long q = q0 + u * EW_T;
+    if (q >= n) continue;
+    const T v = DIM > 0 && fx[u] ? T(0) : cvt<T>(bv[u]);
+    bout[q] = v;
+    z[q] = omega * dv[u] * v;
+  }
   pdl_launch_dependents();
 }
 
+// Result of a V-cycle in float64: on a fixed DOF, where the operator is the
+// identity, two smoothing steps of the input; elsewhere zin (null: out already
+// holds it).
+template <int DIM, typename T>
+__global__ void __launch_bounds__(EW_T)
+    k_vcycle_out(long long n, const T* __restrict__ zin, const double* __restrict__ r, T omega,
+                 const uint8_t* __restrict__ mask, double* __restrict__ out) {
+  const long long q0 = (long long)blockIdx.x * EW_T * EW_U + threadIdx.x;
+  pdl_wait();
+  T zv[EW_U];
+  bool fx[EW_U];
+#pragma unroll
+  for (int u = 0; u < EW_U; ++u) {
+    const long long q = q0 + u * EW_T;
+    if (q >= n) continue;
+    fx[u] = (mask[q / DIM] >> (int)(q % DIM)) & 1u;
+    if (zin) zv[u] = zin[q];
+  }
+#pragma unroll
+  for (int u = 0; u < EW_U; ++u) {
+    const long long q = q0 + u * EW_T;
+    if (q >= n || (!zin && !fx[u])) continue;
+    if (fx[u]) {
+      const T b = (T)r[q], z = omega * b;
+      zv[u] = z + omega * (b - z);
+    }
+    out[q] = (double)zv[u];
+  }
+}
+
 template <typename TIN, typename TOUT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(EW_T)
     k_convert(long long n, const TIN* __restrict__ in, TOUT* __restrict__ out) {
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < n) out[q] = cvt<TOUT>(in[q]);
+  const long long q0 = (long long)blockIdx.x * EW_T * EW_U + threadIdx.x;
+  TIN v[EW_U];
+#pragma unroll
+  for (int u = 0; u < EW_U; ++u)
+    if (q0 + u * EW_T < n) v[u] = in[q0 + u * EW_T];
+#pragma unroll
+  for (int u = 0; u < EW_U; ++u)
+    if (q0 + u * EW_T < n) out[q0 + u * EW_T] = cvt<TOUT>(v[u]);
 }
 
 // ---------------------------------------------------------------------------
@@ -341,26 +396,24 @@ __global__ void __launch_bounds__(256)
 // Host launchers
 // ---------------------------------------------------------------------------
 template <int DIM, typename T>
-static cudaError_t restrict_t(const GridP& gf, const uint8_t* mf, const GridP& gc,
-                              const uint8_t* mc, const void* rf, void* bc, const void* dinvc,
-                              double omega, void* zc, bool clean, cudaStream_t s) {
+static cudaError_t restrict_t(const GridP& gf, const GridP& gc, const uint8_t* mc, const void* rf,
+                              void* bc, const void* dinvc, double omega, void* zc,
+                              cudaStream_t s) {
   if (gc.nn <= 0) return cudaSuccess;
   const long long pv = (long long)DIM * gc.nnx * gc.nny;
   if (pv >= (1LL << 31) - TVAL || gc.nnz > 65535) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((pv + TVAL - 1) / TVAL), DIM == 3 ? gc.nnz : 1);
-  auto kern = clean ? k_restrict<DIM, T, true> : k_restrict<DIM, T, false>;
-  return launch_pdl(kern, grid, dim3(TVAL), 0, s, gf, mf, gc, mc, (const T*)rf, (T*)bc,
+  return launch_pdl(k_restrict<DIM, T>, grid, dim3(TVAL), 0, s, gf, gc, mc, (const T*)rf, (T*)bc,
                     (const T*)dinvc, T(omega), (T*)zc);
 }
 
-cudaError_t launch_restrict(int dim, int t, const GridP& gf, const uint8_t* mf, const GridP& gc,
-                            const uint8_t* mc, const void* rf, void* bc, const void* dinvc,
-                            double omega, void* zc, bool clean, cudaStream_t s) {
-  if (dim == 2)
-    return t == T_F64 ? restrict_t<2, double>(gf, mf, gc, mc, rf, bc, dinvc, omega, zc, clean, s)
-                      : restrict_t<2, float>(gf, mf, gc, mc, rf, bc, dinvc, omega, zc, clean, s);
-  return t == T_F64 ? restrict_t<3, double>(gf, mf, gc, mc, rf, bc, dinvc, omega, zc, clean, s)
-                    : restrict_t<3, float>(gf, mf, gc, mc, rf, bc, dinvc, omega, zc, clean, s);
+cudaError_t launch_restrict(int dim, int t, const GridP& gf, const GridP& gc, const uint8_t* mc,
+                            const void* rf, void* bc, const void* dinvc, double omega, void* zc,
+                            cudaStream_t s) {
+  if (dim == 2) return t == T_F64 ? restrict_t<2, double>(gf, gc, mc, rf, bc, dinvc, omega, zc, s)
+                                  : restrict_t<2, float>(gf, gc, mc, rf, bc, dinvc, omega, zc, s);
+  return t == T_F64 ? restrict_t<3, double>(gf, gc, mc, rf, bc, dinvc, omega, zc, s)
+                    : restrict_t<3, float>(gf, gc, mc, rf, bc, dinvc, omega, zc, s);
 }
 
 template <int DIM, typename T>
@@ -380,41 +433,54 @@ cudaError_t launch_prolong_add(int dim, int t, const GridP& gf, const uint8_t* m
                     : prolong_t<3, float>(gf, mf, gc, zc, zf, s);
 }
 
+template <typename T, typename TIN>
+static cudaError_t presmooth_t(long long n, const void* bin, void* bout, const void* dinv,
+                               double omega, void* z, cudaStream_t s, int dim,
+                               const uint8_t* mask) {
+  auto kern = !mask      ? k_presmooth<0, T, TIN>
+              : dim == 2 ? k_presmooth<2, T, TIN>
+                         : k_presmooth<3, T, TIN>;
+  return launch_pdl(kern, dim3(nblocks(n, EW_T * EW_U)), dim3(EW_T), 0, s, n, (const TIN*)bin,
+                    (T*)bout, (const T*)dinv, (T)omega, (T*)z, mask);
+}
+
 cudaError_t launch_presmooth(int t, int tin, long long n, const void* bin, void* bout,
-                             const void* dinv, double omega, void* z, cudaStream_t s) {
-  const int nb = nblocks(n, 256);
-  if (t == T_F64) {
-    if (tin != T_F64) return cudaErrorInvalidValue;
-    return launch_pdl(k_presmooth<double, double>, dim3(nb), dim3(256), 0, s, n,
-                      (const double*)bin, (double*)bout, (const double*)dinv, omega, (double*)z);
-  } else if (tin == T_F64) {
-    return launch_pdl(k_presmooth<float, double>, dim3(nb), dim3(256), 0, s, n,
-                      (const double*)bin, (float*)bout, (const float*)dinv, (float)omega, (float*)z);
-  } else if (tin == T_D2) {
-    return launch_pdl(k_presmooth<float, float2>, dim3(nb), dim3(256), 0, s, n,
-                      (const float2*)bin, (float*)bout, (const float*)dinv, (float)omega, (float*)z);
-  } else {
-    return launch_pdl(k_presmooth<float, float>, dim3(nb), dim3(256), 0, s, n,
-                      (const float*)bin, (float*)bout, (const float*)dinv, (float)omega, (float*)z);
-  }
-  return cudaGetLastError();
+                             const void* dinv, double omega, void* z, cudaStream_t s, int dim,
+                             const uint8_t* mask) {
+  if (t == T_F64 && tin == T_F64)
+    return presmooth_t<double, double>(n, bin, bout, dinv, omega, z, s, dim, mask);
+  if (t == T_F32 && tin == T_F64)
+    return presmooth_t<float, double>(n, bin, bout, dinv, omega, z, s, dim, mask);
+  if (t == T_F32 && tin == T_D2)
+    return presmooth_t<float, float2>(n, bin, bout, dinv, omega, z, s, dim, mask);
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_vcycle_out(int dim, int t, long long n, const void* zin, const double* r,
+                              double omega, const uint8_t* mask, double* out, cudaStream_t s) {
+  const dim3 grid(nblocks(n, EW_T * EW_U)), th(EW_T);
+  if (t == T_F64)
+    return launch_pdl(dim == 2 ? k_vcycle_out<2, double> : k_vcycle_out<3, double>, grid, th, 0, s,
+                      n, (const double*)zin, r, omega, mask, out);
+  return launch_pdl(dim == 2 ? k_vcycle_out<2, float> : k_vcycle_out<3, float>, grid, th, 0, s, n,
+                    (const float*)zin, r, (float)omega, mask, out);
 }
 
 cudaError_t launch_convert(int tin, int tout, long long n, const void* in, void* out,
                            cudaStream_t s) {
-  const int nb = nblocks(n, 256);
+  const int nb = nblocks(n, EW_T * EW_U);
   if (tin == T_D2 && tout == T_F32)
-    k_convert<float2, float><<<nb, 256, 0, s>>>(n, (const float2*)in, (float*)out);
+    k_convert<float2, float><<<nb, EW_T, 0, s>>>(n, (const float2*)in, (float*)out);
   else if (tin == T_F32 && tout == T_D2)
-    k_convert<float, float2><<<nb, 256, 0, s>>>(n, (const float*)in, (float2*)out);
+    k_convert<float, float2><<<nb, EW_T, 0, s>>>(n, (const float*)in, (float2*)out);
   else if (tin == T_F64 && tout == T_F32)
-    k_convert<double, float><<<nb, 256, 0, s>>>(n, (const double*)in, (float*)out);
+    k_convert<double, float><<<nb, EW_T, 0, s>>>(n, (const double*)in, (float*)out);
   else if (tin == T_F32 && tout == T_F64)
-    k_convert<float, double><<<nb, 256, 0, s>>>(n, (const float*)in, (double*)out);
+    k_convert<float, double><<<nb, EW_T, 0, s>>>(n, (const float*)in, (double*)out);
   else if (tin == T_F64)
-    k_convert<double, double><<<nb, 256, 0, s>>>(n, (const double*)in, (double*)out);
+    k_convert<double, double><<<nb, EW_T, 0, s>>>(n, (const double*)in, (double*)out);
   else
-    k_convert<float, float><<<nb, 256, 0, s>>>(n, (const float*)in, (float*)out);
+    k_convert<float, float><<<nb, EW_T, 0, s>>>(n, (const float*)in, (float*)out);
   return cudaGetLastError();
 }
 

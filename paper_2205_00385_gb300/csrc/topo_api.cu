@@ -874,11 +874,11 @@ static double vbytes_coarse(long long nc, int ta, int t) {
          2.0 * (t == T_F64 ? 8.0 : 4.0) * (double)nc;
 }
 
-// clean: the right-hand side is zero on every fixed DOF (the solver's CG
-// residual), so the finest level's vectors are too and its float32 operator
-// needs to mask only the fixed rows' outputs.
+// The right-hand side is zero on every fixed DOF (the solver's residual, or
+// cleared by the presmoothing), so the finest level's vectors are too and its
+// operators need to mask only the fixed rows' outputs.
 static to_status vcycle(to_ctx* c, const void* rin, int rin_t, void* zout, int zt,
-                        bool pre = false, bool clean = false) {
+                        bool pre = false) {
   cudaStream_t s = c->stream;
   const int t = mg_t(c);
   const int L = c->L;
@@ -895,19 +895,18 @@ static to_status vcycle(to_ctx* c, const void* rin, int rin_t, void* zout, int z
   {
     ApplyArgs a = fine_args(c, TO_OP_K, t, t, t, lv[0].z, lv[0].r, lv[0].b, lv[0].dinv,
                             EPI_RESID);
-    a.clean_inputs = clean;
+    a.clean_inputs = true;
     vb += apply_bytes(a);
     if ((st = run_op(c, a, "resid 0")) != TO_OK) return st;
   }
   // restriction into level l also pre-smooths level l from a zero guess
-  // (except on the coarsest level, which is solved exactly).  The residual of
-  // a coarse level is zero on its fixed DOFs (its right-hand side and
-  // zero-guess smoothing are), that of the finest level when the input is.
+  // (except on the coarsest level, which is solved exactly).  Every level's
+  // residual is zero on its fixed DOFs: its right-hand side and zero-guess
+  // smoothing are.
   auto restrict_into = [&](int l) {
     const bool smooth = l < L - 1;
-    return launch_restrict(c->dim, t, lv[l - 1].g, lv[l - 1].mask, lv[l].g, lv[l].mask,
-                           lv[l - 1].r, lv[l].b, smooth ? lv[l].dinv : nullptr, 0.6,
-                           smooth ? lv[l].z : nullptr, clean || l >= 2, s);
+    return launch_restrict(c->dim, t, lv[l - 1].g, lv[l].g, lv[l].mask, lv[l - 1].r, lv[l].b,
+                           smooth ? lv[l].dinv : nullptr, 0.6, smooth ? lv[l].z : nullptr, s);
   };
   // levels lf .. L-1 (lf = 0: none) run as one fused cluster launch
   const int lf = c->fuse_coarse ? c->vf_l0 : 0;
@@ -918,7 +917,7 @@ static to_status vcycle(to_ctx* c, const void* rin, int rin_t, void* zout, int z
   for (int l = 1; l < L - 1; ++l) {
     if (lf && l >= lf) break;
     ApplyArgs a = coarse_args(c, l, lv[l].z, lv[l].r, lv[l].b, EPI_RESID);
-    a.clean_inputs = clean;
+    a.clean_inputs = true;
     vb += apply_bytes(a);
     if ((st = run_op(c, a, "resid l")) != TO_OK) return st;
     if (lf && l + 1 == lf) break;
@@ -958,7 +957,7 @@ static to_status vcycle(to_ctx* c, const void* rin, int rin_t, void* zout, int z
                                  lv[l].z, s), "prolong l");
     vb += vbytes_prolong(lv[l].n, lv[l + 1].n, t);
     ApplyArgs a = coarse_args(c, l, lv[l].z, lv[l].z2, lv[l].b, EPI_SMOOTH);
-    a.clean_inputs = clean;
+    a.clean_inputs = true;
     vb += apply_bytes(a);
     if ((st = run_op(c, a, "postsmooth l")) != TO_OK) return st;
   }
@@ -967,7 +966,7 @@ static to_status vcycle(to_ctx* c, const void* rin, int rin_t, void* zout, int z
   vb += vbytes_prolong(lv[0].n, lv[1].n, t);
   ApplyArgs a = fine_args(c, TO_OP_K, t, t, zt, lv[0].z, zout, lv[0].b, lv[0].dinv,
                           EPI_SMOOTH);
-  a.clean_inputs = clean;
+  a.clean_inputs = true;
   vb += apply_bytes(a);
   ps.bytes = vb;
   c->vcycle_bytes = vb;
@@ -1000,7 +999,7 @@ static to_status vcycle_graphed(to_ctx* c, const void* rin, int rin_t, void* zou
     to_status st = TO_OK;
     cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      st = vcycle(c, rin, rin_t, zout, zt, pre, true);
+      st = vcycle(c, rin, rin_t, zout, zt, pre);
       const cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &graph);
       if (e == cudaSuccess) e = e2;
     }
@@ -1130,10 +1129,28 @@ to_status to_vcycle(to_ctx* c, const double* r, double* z) {
     to_status st = build_hierarchy(c);
     if (st != TO_OK) return st;
   }
-  if (!c->mixed) return vcycle(c, r, T_F64, z, T_F64);
-  to_status st = vcycle(c, r, T_F64, c->lv[0].z2, T_F32);
+  // The cycle runs on the input with its fixed DOFs cleared (what they hold
+  // reaches no free DOF), so its operators mask outputs only; their own rows
+  // are added at the end.
+  cudaStream_t s = c->stream;
+  const int t = mg_t(c);
+  LevelBuf& l0 = c->lv[0];
+  to_status st;
+  LAUNCH(c, launch_presmooth(t, T_F64, c->n, r, l0.b, l0.dinv, 0.6, l0.z, s, c->dim, l0.mask),
+         "presmooth 0");
+  // mixed: the solver's captured cycle (its buffers are the context's own)
+  // unless the caller captures or times single kernels
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CUDA_TRY(c, cudaStreamIsCapturing(s, &cap), "capture status");
+  const bool graphed = c->mixed && cap == cudaStreamCaptureStatusNone &&
+                       !(c->prof_mask & ~(1u << PK_VCYCLE));
+  if (graphed)
+    st = vcycle_graphed(c, c->r, T_D2, l0.z2, T_F32, true);
+  else
+    st = vcycle(c, nullptr, t, c->mixed ? l0.z2 : (void*)z, t, true);
   if (st != TO_OK) return st;
-  LAUNCH(c, launch_convert(T_F32, T_F64, c->n, c->lv[0].z2, z, c->stream), "convert");
+  LAUNCH(c, launch_vcycle_out(c->dim, t, c->n, c->mixed ? l0.z2 : nullptr, r, 0.6, l0.mask, z, s),
+         "V-cycle result");
   return TO_OK;
 }
 
