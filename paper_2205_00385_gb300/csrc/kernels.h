@@ -187,8 +187,8 @@ cudaError_t launch_dot(long long n, const double* a, const double* b, double* pa
                        unsigned* counter, double* out, cudaStream_t s);
 // alpha = scal[num] / scal[den]; x += alpha p; r -= alpha q; scal[rr] = r.r
 cudaError_t launch_cg_xr(long long n, double* x, double* r, const double* p, const double* q,
-                         double* scal, int num, int den, int rr, double* partials,
-                         unsigned* counter, cudaStream_t s, double* host_rr = nullptr);
+                         double* scal, double* partials, unsigned* counter, cudaStream_t s,
+                         double* host_rr);
 // beta = scal[num] / scal[den]; p = z + beta p
 cudaError_t launch_cg_p(long long n, double* p, const double* z, const double* scal, int num,
                         int den, cudaStream_t s);
@@ -253,14 +253,12 @@ cudaError_t launch_cg_q2_df(const GridP& g, const uint8_t* mask, const double* k
 // the workspace, 16-byte aligned): out = a . b
 cudaError_t launch_dot_d2f(long long n, const void* a, const float* b, double* partials,
                            unsigned* counter, double* out, cudaStream_t s);
-// x += alpha p, r -= alpha q, scal[rr] = |r|^2 with alpha = scal[num]/scal[den];
-// b = float(r), zpre = omega dinv b (the next V-cycle's right-hand side and
-// pre-smoothing from zero); host_rr (may be null): a device-accessible pointer
-// to pinned host memory that also receives |r|^2
+// the CG update (k_cg_xr) on pairs; also b = float(r), zpre = omega dinv b (the
+// next V-cycle's right-hand side and pre-smoothing from zero)
 cudaError_t launch_cg_xr_d2(long long n, void* x, void* r, const void* p, const float* q,
-                            double* scal, int num, int den, int rr, double* partials,
-                            unsigned* counter, float* b, float* zpre, const float* dinv,
-                            double omega, cudaStream_t s, double* host_rr = nullptr);
+                            double* scal, double* partials, unsigned* counter, float* b,
+                            float* zpre, const float* dinv, double omega, cudaStream_t s,
+                            double* host_rr);
 // p = z + beta p (num < 0: p = z), beta = scal[num]/scal[den]; p32 = float(p)
 cudaError_t launch_cg_p_d2(long long n, void* p, float* p32, const float* z, const double* scal,
                            int num, int den, cudaStream_t s);

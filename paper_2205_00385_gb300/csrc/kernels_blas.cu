@@ -27,15 +27,17 @@ __global__ void __launch_bounds__(RED_THREADS)
   }
 }
 
-// host_rr (may be null): pinned host memory mapped into the device's
-// address space that also receives |r|^2
+// alpha = scal[S_RZ1] / scal[S_PQ]; x += alpha p, r -= alpha q, scal[S_RR] =
+// |r|^2; scal[S_RZ0] = scal[S_RZ1].  host_rr: pinned host memory mapped into the
+// device's address space that receives |r|^2 and then the number of updates
+// so far (scal[S_CG_COUNT]).
 __global__ void __launch_bounds__(RED_THREADS)
     k_cg_xr(long long n, double* __restrict__ x, double* __restrict__ r,
-            const double* __restrict__ p, const double* __restrict__ q, double* scal, int num,
-            int den, int rr, double* partials, unsigned* counter, double* host_rr) {
+            const double* __restrict__ p, const double* __restrict__ q, double* scal,
+            double* partials, unsigned* counter, double* host_rr) {
   __shared__ double sh[32], s_alpha;
   pdl_wait();
-  if (threadIdx.x == 0) s_alpha = scal[num] / scal[den];   // one division per block
+  if (threadIdx.x == 0) s_alpha = scal[S_RZ1] / scal[S_PQ];   // one division per block
   __syncthreads();
   const double alpha = s_alpha;
   double v[1] = {0.0};
@@ -51,13 +53,7 @@ __global__ void __launch_bounds__(RED_THREADS)
   if (publish_partials<1>(v, partials, counter)) {
     double o[1];
     finish_sum<1>(partials, counter, o, sh);
-    if (threadIdx.x == 0) {
-      scal[rr] = o[0];
-      if (host_rr) {
-        *reinterpret_cast<volatile double*>(host_rr) = o[0];
-        __threadfence_system();
-      }
-    }
+    if (threadIdx.x == 0) cg_publish(scal, o[0], host_rr);
   }
 }
 
@@ -370,10 +366,10 @@ cudaError_t launch_dot(long long n, const double* a, const double* b, double* pa
 }
 
 cudaError_t launch_cg_xr(long long n, double* x, double* r, const double* p, const double* q,
-                         double* scal, int num, int den, int rr, double* partials,
-                         unsigned* counter, cudaStream_t s, double* host_rr) {
-  return launch_pdl(k_cg_xr, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n, x, r, p, q, scal, num, den,
-                    rr, partials, counter, host_rr);
+                         double* scal, double* partials, unsigned* counter, cudaStream_t s,
+                         double* host_rr) {
+  return launch_pdl(k_cg_xr, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n, x, r, p, q, scal,
+                    partials, counter, host_rr);
 }
 
 cudaError_t launch_cg_p(long long n, double* p, const double* z, const double* scal, int num,

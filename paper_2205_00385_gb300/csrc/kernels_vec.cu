@@ -590,25 +590,22 @@ __global__ void __launch_bounds__(VEC_T)
   if (grid_sum_df(w, sh, tot, partials, counter) && threadIdx.x == 0) *out = tot[0];
 }
 
-// alpha = scal[num] / scal[den]; x += alpha p; r -= alpha q; scal[rr] = |r|^2.
-// It also starts the next V-cycle: b = r rounded to float32 and
-// zpre = omega dinv b (its pre-smoothing from a zero guess), the values the
-// V-cycle's first kernel would compute.
-// With host_rr set, |r|^2 is also written there (pinned host memory mapped
-// into the device's address space), so the host reads it after an event on
-// the stream without a copy between this kernel and the next.
+// The CG update of kernels_blas.cu (k_cg_xr) on pairs.  It also starts the
+// next V-cycle: b = r rounded to float32 and zpre = omega dinv b (its
+// pre-smoothing from a zero guess), the values the V-cycle's first kernel
+// would compute.
 constexpr int CG_U = 2;
 __global__ void __launch_bounds__(VEC_T)
     k_cg_xr_d2(long long n, float2* __restrict__ x, float2* __restrict__ r,
-               const float2* __restrict__ p, const float* __restrict__ q, double* scal, int num,
-               int den, int rr, double* partials, unsigned* counter, float* __restrict__ b,
+               const float2* __restrict__ p, const float* __restrict__ q, double* scal,
+               double* partials, unsigned* counter, float* __restrict__ b,
                float* __restrict__ zpre, const float* __restrict__ dinv, float omega,
                double* host_rr) {
   using Rg = Ar<float2>;
   __shared__ double sh[1][VEC_W], tot[1];
   __shared__ dfl s_alpha;
   pdl_wait();
-  if (threadIdx.x == 0) s_alpha = split_d(scal[num] / scal[den]);
+  if (threadIdx.x == 0) s_alpha = split_d(scal[S_RZ1] / scal[S_PQ]);
   __syncthreads();
   const dfl al = s_alpha, mal = {-al.h, -al.l};
   dfl v[2] = {{0.f, 0.f}, {0.f, 0.f}};
@@ -649,13 +646,8 @@ __global__ void __launch_bounds__(VEC_T)
       });
   pdl_launch_dependents();
   const dfl w[1] = {df_add(df_norm(v[0]), df_norm(v[1]))};
-  if (grid_sum_df(w, sh, tot, partials, counter) && threadIdx.x == 0) {
-    scal[rr] = tot[0];
-    if (host_rr) {
-      *reinterpret_cast<volatile double*>(host_rr) = tot[0];
-      __threadfence_system();
-    }
-  }
+  if (grid_sum_df(w, sh, tot, partials, counter) && threadIdx.x == 0)
+    cg_publish(scal, tot[0], host_rr);
 }
 
 // p = z + beta p (beta = scal[num]/scal[den], or p = z when num < 0);
@@ -946,11 +938,11 @@ cudaError_t launch_dot_d2f(long long n, const void* a, const float* b, double* p
 }
 
 cudaError_t launch_cg_xr_d2(long long n, void* x, void* r, const void* p, const float* q,
-                            double* scal, int num, int den, int rr, double* partials,
-                            unsigned* counter, float* b, float* zpre, const float* dinv,
-                            double omega, cudaStream_t s, double* host_rr) {
+                            double* scal, double* partials, unsigned* counter, float* b,
+                            float* zpre, const float* dinv, double omega, cudaStream_t s,
+                            double* host_rr) {
   return launch_pdl(k_cg_xr_d2, pair2_grid(n, 1), dim3(VEC_T), 0, s, n, (float2*)x, (float2*)r,
-                    (const float2*)p, q, scal, num, den, rr, partials, counter, b, zpre, dinv,
+                    (const float2*)p, q, scal, partials, counter, b, zpre, dinv,
                     (float)omega, host_rr);
 }
 

@@ -4,6 +4,7 @@
 // bookkeeping (level geometry, PARM ring position, iteration counts); every
 // arithmetic step of the solver path runs in the library's kernels.  Device
 // memory comes exclusively from the caller's workspace.
+#include <atomic>
 #include <cmath>
 #include <map>
 #include <mutex>
@@ -14,6 +15,7 @@
 
 #include <algorithm>
 #include <string>
+#include <thread>
 
 #include "kernels.h"
 
@@ -503,7 +505,6 @@ to_status to_mesh_init(const to_mesh_desc* desc, const uint8_t* fixed_mask, cons
   c->oc_eta = 0.5;
   c->host_rr = nullptr;
   c->host_rr_dev = nullptr;
-  c->rr_event = nullptr;
   c->cap_stream = nullptr;
   if (!make_stencil(c->dim, desc->rmin, &c->stencil)) {
     delete c;
@@ -629,7 +630,6 @@ void to_destroy(to_ctx* ctx) {
   for (int q = 0; q < ctx->n_vgraph; ++q) cudaGraphExecDestroy(ctx->vgraph[q].exec);
   batch_forget(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
-  if (ctx->rr_event) cudaEventDestroy(ctx->rr_event);
   if (ctx->host_rr) cudaFreeHost(ctx->host_rr);
   delete ctx;
 }
@@ -978,13 +978,13 @@ static to_status vcycle(to_ctx* c, const void* rin, int rin_t, void* zout, int z
 // in float64), so it is captured once per (input, output, precision,
 // coefficients) as a CUDA graph and replayed: one launch per preconditioner
 // application instead of one per kernel, with no host gaps between kernels.
-static to_status vcycle_graphed(to_ctx* c, const void* rin, int rin_t, void* zout, int zt,
-                                bool pre = false) {
-  const void* coef = mg_t(c) == T_F64 ? (const void*)c->E64 : (const void*)c->E32;
+template <typename Body>
+static to_status run_graphed(to_ctx* c, const void* rin, const void* zout, const void* coef,
+                             int kind, bool pre, const Body& body) {
   to_ctx::VGraph* vg = nullptr;
   for (int q = 0; q < c->n_vgraph; ++q) {
     to_ctx::VGraph& v = c->vgraph[q];
-    if (v.rin == rin && v.zout == zout && v.zt == zt && v.coef == coef && v.pre == pre) vg = &v;
+    if (v.rin == rin && v.zout == zout && v.kind == kind && v.coef == coef && v.pre == pre) vg = &v;
   }
   if (!vg) {
     if (!c->cap_stream)
@@ -999,7 +999,7 @@ static to_status vcycle_graphed(to_ctx* c, const void* rin, int rin_t, void* zou
     to_status st = TO_OK;
     cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      st = vcycle(c, rin, rin_t, zout, zt, pre);
+      st = body();
       const cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &graph);
       if (e == cudaSuccess) e = e2;
     }
@@ -1012,18 +1012,25 @@ static to_status vcycle_graphed(to_ctx* c, const void* rin, int rin_t, void* zou
     if (graph) cudaGraphDestroy(graph);
     if (st != TO_OK) return st;
     if (e != cudaSuccess) return cuda_fail(c, "V-cycle graph", e);
-    if (c->n_vgraph == 4) {
+    if (c->n_vgraph == to_ctx::MAX_VGRAPH) {
       cudaGraphExecDestroy(c->vgraph[0].exec);
-      for (int q = 1; q < 4; ++q) c->vgraph[q - 1] = c->vgraph[q];
-      c->n_vgraph = 3;
+      for (int q = 1; q < c->n_vgraph; ++q) c->vgraph[q - 1] = c->vgraph[q];
+      --c->n_vgraph;
     }
     vg = &c->vgraph[c->n_vgraph++];
-    *vg = to_ctx::VGraph{rin, zout, coef, zt, pre, exec, captured, c->vcycle_bytes};
+    *vg = to_ctx::VGraph{rin, zout, coef, kind, pre, exec, captured, c->vcycle_bytes};
   }
   ProfScope ps(c, PK_VCYCLE, vg->bytes);
   CUDA_TRY(c, cudaGraphLaunch(vg->exec, c->stream), "V-cycle graph launch");
   c->launches += vg->launches;
   return TO_OK;
+}
+
+static to_status vcycle_graphed(to_ctx* c, const void* rin, int rin_t, void* zout, int zt,
+                                bool pre = false) {
+  const void* coef = mg_t(c) == T_F64 ? (const void*)c->E64 : (const void*)c->E32;
+  return run_graphed(c, rin, zout, coef, zt, pre,
+                     [&] { return vcycle(c, rin, rin_t, zout, zt, pre); });
 }
 
 static to_status read_scalar(to_ctx* c, const double* dev, double* host) {
@@ -1188,8 +1195,8 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
   if (c->hier_stale && (st = build_hierarchy(c)) != TO_OK) return st;
   if (!c->host_rr) {
     // 64 bytes of pinned host memory per context, mapped into the device's
-    // address space: the CG update kernel writes |r|^2 there itself and the
-    // host waits on an event recorded after it
+    // address space: the CG update kernel writes |r|^2 there itself, then its
+    // own count, which the host waits for
     void* h = nullptr;
     CUDA_TRY(c, cudaHostAlloc(&h, 64, cudaHostAllocMapped), "pinned residual slot");
     c->host_rr = static_cast<double*>(h);
@@ -1197,15 +1204,18 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
     CUDA_TRY(c, cudaHostGetDevicePointer(&d, h, 0), "mapped residual slot");
     c->host_rr_dev = static_cast<double*>(d);
   }
-  if (!c->rr_event)
-    CUDA_TRY(c, cudaEventCreateWithFlags(&c->rr_event, cudaEventDisableTiming), "rr event");
+  // no update of an earlier solve is in flight (each ends synchronised)
+  c->host_rr[1] = 0.0;
+  CUDA_TRY(c, cudaMemsetAsync(c->scal + S_CG_COUNT, 0, 8, s), "reset count");
   const long long n = c->n;
   // Mixed path: the iterate x, r and p are double-float pairs (x in the
   // otherwise unused float64 z buffer); the operator and the V-cycle work on
   // float32 shadows (p32 -> q32, z32); dot products are double-float.
-  // FP64 path: everything float64, x = u.
+  // FP64 path: everything float64, the iterate in the scratch vector t.
+  // Every vector is the context's own, so that captured iterations serve
+  // whatever u a call brings.
   const bool mixed = c->mixed;
-  double* x = mixed ? c->z : u;
+  double* x = mixed ? c->z : c->t;
   const bool warm = (flags & TO_SOLVE_WARM_START) != 0;
   if (mixed && warm) {
     LAUNCH(c, launch_vconvert(n, V_F64, u, V_DF2, x, s), "split u");
@@ -1216,6 +1226,7 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
   } else if (!warm) {
     CUDA_TRY(c, cudaMemsetAsync(x, 0, n * 8, s), "zero x");
   } else {
+    LAUNCH(c, launch_copy(n, u, x, s), "copy u");
     LAUNCH(c, launch_zero_fixed(c->nn, c->dim, c->lv[0].mask, V_F64, x, s), "clear fixed");
   }
   // r = f - K x with the float64-accurate operator (the true residual)
@@ -1236,85 +1247,132 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
   // mixed path: the CG update also writes the next V-cycle's right-hand side
   // and pre-smoothing (lv[0].b, lv[0].z); a true residual invalidates them
   bool pre = false;
-  auto precondition = [&](int slot) -> to_status {
+  // (the enqueuing steps below run on c->stream, which is the capture stream
+  // while an iteration is being captured)
+  auto dot_rz = [&]() -> to_status {
+    if (mixed)
+      LAUNCH(c, launch_dot_d2f(n, c->r, z32, c->partials, c->counters + C_DOT, c->scal + S_RZ1,
+                               c->stream), "rz");
+    else
+      LAUNCH(c, launch_dot(n, c->r, c->z, c->partials, c->counters + C_DOT, c->scal + S_RZ1,
+                           c->stream), "rz");
+    return TO_OK;
+  };
+  auto precondition = [&]() -> to_status {
+    const to_status e = mixed ? vcycle_graphed(c, c->r, T_D2, z32, T_F32, pre)
+                              : vcycle_graphed(c, c->r, T_F64, c->z, T_F64);
+    return e != TO_OK ? e : dot_rz();
+  };
+  // p = z + beta p, beta = scal[S_RZ1] / scal[S_RZ0] (first: p = z)
+  auto update_p = [&](bool first) -> to_status {
+    if (mixed)
+      LAUNCH(c, launch_cg_p_d2(n, c->p, c->p32, z32, c->scal, first ? -1 : S_RZ1, S_RZ0, c->stream),
+             "p update");
+    else if (first)
+      LAUNCH(c, launch_copy(n, c->z, c->p, c->stream), "p = z");
+    else
+      LAUNCH(c, launch_cg_p(n, c->p, c->z, c->scal, S_RZ1, S_RZ0, c->stream), "p update");
+    return TO_OK;
+  };
+  // Precision escalation (mixed path, 3D; in 2D, where a float32 K p loses
+  // percents on the longer spans, q is formed in double-float throughout):
+  // q = K p in float32 carries ~1e-4 relative error on smooth search
+  // directions (K cancels by 1e3-1e4 there), and on some designs CG
+  // stagnates on it, the recursive and true residuals stuck together.
+  // Healthy convergence gains >= 10x in 16 iterations; when the residual
+  // fails to halve over 16 iterations, the rest of the solve forms q with the
+  // double-float operator (then rounded to float32, which loses nothing to
+  // cancellation) and CG restarts from the true residual.
+  bool accurate_q = false;
+  // q = K p; alpha = rz / pq; x, r and |r|^2 (which the update kernel also writes
+  // to the host); rz becomes the old one of the next direction
+  auto advance = [&]() -> to_status {
     to_status e;
-    if (mixed) {
-      if ((e = vcycle_graphed(c, c->r, T_D2, z32, T_F32, pre)) != TO_OK) return e;
-      LAUNCH(c, launch_dot_d2f(n, c->r, z32, c->partials, c->counters + C_DOT, c->scal + slot, s),
-             "rz");
+    if (mixed && c->dim == 2) {
+      LAUNCH(c, launch_cg_q2_df(c->lv[0].g, c->lv[0].mask, c->KE64, c->E64, c->p, c->q32,
+                                c->springs, c->partials, c->counters + C_DOT, c->scal + S_PQ,
+                                c->stream), "q = K p, pq");
+    } else if (mixed && accurate_q) {
+      if ((e = apply_accurate_vec(c, TO_OP_K, c->p, c->t, EPI_APPLY)) != TO_OK) return e;
+      LAUNCH(c, launch_convert(T_D2, T_F32, n, c->t, c->q32, c->stream), "q to float32");
     } else {
-      if ((e = vcycle_graphed(c, c->r, T_F64, c->z, T_F64)) != TO_OK) return e;
-      LAUNCH(c, launch_dot(n, c->r, c->z, c->partials, c->counters + C_DOT, c->scal + slot, s),
-             "rz");
+      ApplyArgs a = mixed ? fine_args(c, TO_OP_K, T_F32, T_F32, T_F32, c->p32, c->q32, nullptr,
+                                      nullptr, EPI_APPLY)
+                          : fine_args(c, TO_OP_K, T_F64, T_F64, T_F64, c->p, c->q, nullptr, nullptr,
+                                      EPI_APPLY);
+      a.clean_inputs = true;   // p is zero on the fixed DOFs
+      if ((e = run_op(c, a, "q = K p")) != TO_OK) return e;
+    }
+    if (mixed) {
+      if (c->dim == 3)
+        LAUNCH(c, launch_dot_d2f(n, c->p, c->q32, c->partials, c->counters + C_DOT, c->scal + S_PQ,
+                                 c->stream), "pq");
+      LAUNCH(c, launch_cg_xr_d2(n, x, c->r, c->p, c->q32, c->scal, c->partials,
+                                c->counters + C_UPD, static_cast<float*>(c->lv[0].b),
+                                static_cast<float*>(c->lv[0].z),
+                                static_cast<const float*>(c->lv[0].dinv), 0.6, c->stream,
+                                c->host_rr_dev), "x, r update");
+    } else {
+      LAUNCH(c, launch_dot(n, c->p, c->q, c->partials, c->counters + C_DOT, c->scal + S_PQ,
+                           c->stream), "pq");
+      LAUNCH(c, launch_cg_xr(n, x, c->r, c->p, c->q, c->scal, c->partials, c->counters + C_UPD,
+                             c->stream, c->host_rr_dev), "x, r update");
     }
     return TO_OK;
   };
+  // An iteration in the middle of a solve -- direction, product, update,
+  // V-cycle, rz -- as one captured graph: between two graphs the device idles
+  // some microseconds, so V-cycles captured alone pay that twice.
+  auto iteration = [&]() -> to_status {
+    const void* coef = mixed && c->dim == 3 ? (const void*)c->E32 : (const void*)c->E64;
+    return run_graphed(c, x, mixed ? (void*)z32 : (void*)c->z, coef, to_ctx::CG_ITERATION, mixed,
+                       [&]() -> to_status {
+                         to_status e;
+                         if ((e = update_p(false)) != TO_OK || (e = advance()) != TO_OK) return e;
+                         e = mixed ? vcycle(c, c->r, T_D2, z32, T_F32, true)
+                                   : vcycle(c, c->r, T_F64, c->z, T_F64);
+                         return e != TO_OK ? e : dot_rz();
+                       });
+  };
+  // |r|^2 of update number it, from the mapped slot: the kernel writes it, then
+  // the count.  The stream is asked now and then whether it still runs.
+  auto wait_rr = [&](int count, double* out) -> to_status {
+    const volatile double* slot = c->host_rr;
+    for (long long spin = 1; slot[1] != (double)count; ++spin) {
+      if (spin % 64 == 0) std::this_thread::yield();
+      if (spin % 16384) continue;
+      const cudaError_t e = cudaStreamQuery(s);
+      if (e == cudaErrorNotReady) continue;
+      if (e != cudaSuccess) return cuda_fail(c, "CG iteration", e);
+      if (slot[1] != (double)count) return fail(c, TO_E_CUDA, "CG update left no residual");
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    *out = slot[0];
+    return TO_OK;
+  };
   if (!conv) {
-    if ((st = precondition(S_RZ0)) != TO_OK) return st;
-    if (mixed)
-      LAUNCH(c, launch_cg_p_d2(n, c->p, c->p32, z32, c->scal, -1, 0, s), "p = z");
-    else
-      LAUNCH(c, launch_copy(n, c->z, c->p, s), "p = z");
-    int cur = S_RZ0, nxt = S_RZ1;
-    // Precision escalation (mixed path, 3D; in 2D, where a float32 K p loses
-    // percents on the longer spans, q is formed in double-float throughout):
-    // q = K p in float32 carries ~1e-4 relative error on smooth search
-    // directions (K cancels by 1e3-1e4 there), and on some designs CG
-    // stagnates on it, the recursive and true residuals stuck together.  Healthy convergence gains >= 10x in
-    // 16 iterations; when the residual fails to halve over 16 iterations,
-    // the rest of the solve forms q with the double-float operator (then
-    // rounded to float32, which loses nothing to cancellation) and CG
-    // restarts from the true residual.
-    bool accurate_q = false;
+    if ((st = precondition()) != TO_OK) return st;
     double rel_window = rel;
     int it_window = 0;
+    bool fresh = true, restart = true;   // z is of the current r; p = z
     for (it = 1; it <= maxit; ++it) {
-      if (mixed && c->dim == 2) {
-        LAUNCH(c, launch_cg_q2_df(c->lv[0].g, c->lv[0].mask, c->KE64, c->E64, c->p, c->q32,
-                                  c->springs, c->partials, c->counters + C_DOT, c->scal + S_PQ, s),
-               "q = K p, pq");
-      } else if (mixed && accurate_q) {
-        if ((st = apply_accurate_vec(c, TO_OP_K, c->p, c->t, EPI_APPLY)) != TO_OK) return st;
-        LAUNCH(c, launch_convert(T_D2, T_F32, n, c->t, c->q32, s), "q to float32");
-      } else if (mixed) {
-        ApplyArgs a = fine_args(c, TO_OP_K, T_F32, T_F32, T_F32, c->p32, c->q32, nullptr,
-                                nullptr, EPI_APPLY);
-        a.clean_inputs = true;   // p is zero on the fixed DOFs
-        if ((st = run_op(c, a, "q = K p")) != TO_OK) return st;
-      }
-      if (mixed) {
-        if (c->dim == 3)
-          LAUNCH(c, launch_dot_d2f(n, c->p, c->q32, c->partials, c->counters + C_DOT,
-                                   c->scal + S_PQ, s), "pq");
-        LAUNCH(c, launch_cg_xr_d2(n, x, c->r, c->p, c->q32, c->scal, cur, S_PQ, S_RR,
-                                  c->partials, c->counters + C_UPD,
-                                  static_cast<float*>(c->lv[0].b), static_cast<float*>(c->lv[0].z),
-                                  static_cast<const float*>(c->lv[0].dinv), 0.6, s,
-                                  c->host_rr_dev),
-               "x, r update");
-        pre = true;
+      // The next preconditioner application is enqueued before the host waits
+      // for |r|^2: the V-cycle runs while the host reads it and decides.  It
+      // writes only its own scratch and scal[S_RZ1], so when the loop stops
+      // (or a true residual replaces r) its result is discarded (or
+      // recomputed) and the iterates are the same as with the read first.
+      if (fresh && !restart && it < maxit && !accurate_q && !c->prof_mask) {
+        if ((st = iteration()) != TO_OK) return st;
       } else {
-        ApplyArgs a = fine_args(c, TO_OP_K, T_F64, T_F64, T_F64, c->p, c->q, nullptr, nullptr,
-                                EPI_APPLY);
-        a.clean_inputs = true;   // p is zero on the fixed DOFs
-        if ((st = run_op(c, a, "q = K p")) != TO_OK) return st;
-        LAUNCH(c, launch_dot(n, c->p, c->q, c->partials, c->counters + C_DOT, c->scal + S_PQ, s),
-               "pq");
-        LAUNCH(c, launch_cg_xr(n, x, c->r, c->p, c->q, c->scal, cur, S_PQ, S_RR, c->partials,
-                               c->counters + C_UPD, s, c->host_rr_dev), "x, r update");
+        if (!fresh && (st = precondition()) != TO_OK) return st;
+        if ((st = update_p(restart)) != TO_OK || (st = advance()) != TO_OK) return st;
+        pre = mixed;
+        if (it < maxit && (st = precondition()) != TO_OK) return st;
       }
-      // |r|^2 goes to the host, and the next preconditioner application is
-      // enqueued before the host waits for it: the V-cycle runs while the
-      // host reads the residual and decides.  The preconditioner writes only
-      // its own scratch and scal[nxt], so when the loop stops (or a true
-      // residual replaces r) its result is discarded (or recomputed) and
-      // the iterates are the same as with the read first.
-      // (the update kernel writes it into the mapped host slot itself)
-      CUDA_TRY(c, cudaEventRecord(c->rr_event, s), "rr event");
-      bool fresh = it < maxit;
-      if (fresh && (st = precondition(nxt)) != TO_OK) return st;
-      CUDA_TRY(c, cudaEventSynchronize(c->rr_event), "wait rr");
-      rr = *reinterpret_cast<volatile double*>(c->host_rr);
+      pre = mixed;
+      fresh = it < maxit;
+      restart = false;
+      if ((st = wait_rr(it, &rr)) != TO_OK) return st;
       rel = sqrt(rr) / c->fnorm;
       if (!isfinite(rel)) return fail(c, TO_E_SINGULAR, "CG breakdown (non-finite residual)");
       // Reliable updates: with a float32 operator the recursive residual
@@ -1325,7 +1383,6 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
       // recursive one the recursion has drifted (its directions were built
       // for a different residual), and CG restarts from the true residual
       // (p = z).
-      bool restart = false;
       bool escalate = false;
       if (mixed && c->dim == 3 && !accurate_q && it - it_window >= 16) {
         escalate = rel > 0.5 * rel_window;
@@ -1347,19 +1404,12 @@ to_status to_mgcg_solve(to_ctx* c, double rtol, int32_t maxit, int32_t flags, do
         conv = true;
         break;
       }
-      if (it == maxit) break;
-      if (!fresh && (st = precondition(nxt)) != TO_OK) return st;
-      if (mixed)
-        LAUNCH(c, launch_cg_p_d2(n, c->p, c->p32, z32, c->scal, restart ? -1 : nxt, cur, s),
-               "p update");
-      else
-        LAUNCH(c, launch_cg_p(n, c->p, c->z, c->scal, nxt, cur, s), "p update");
-      std::swap(cur, nxt);
     }
     if (it > maxit) it = maxit;
     // the iterate back to float64 (untouched when no step was taken)
     if (mixed) LAUNCH(c, launch_vconvert(n, V_DF2, x, V_F64, u, s), "widen x");
   }
+  if (!mixed) LAUNCH(c, launch_copy(n, x, u, s), "copy x");
   if (iters) *iters = it;
   if (relres) *relres = rel;
   if ((st = check_status(c)) != TO_OK) return st;

@@ -115,6 +115,7 @@ enum Slot {
   S_NRM0 = 13, S_NRM1 = 14, S_FNORM2 = 15, S_FLAG = 16,
   // OC search: volumes and factors lambda^-eta at the bracket's ends, the
   // sweep's multipliers and their factors
+  S_CG_COUNT = 21,   // updates of the current solve
   S_OC_V1 = 17, S_OC_V2 = 18, S_OC_S1 = 19, S_OC_S2 = 20, S_OC_NPT = 8, S_OC_PT = 24, S_OC_SP = S_OC_PT + S_OC_NPT,
   S_NSLOTS = 64
 };
@@ -190,6 +191,21 @@ __device__ __forceinline__ void block_max(double (&v)[NV], double* sh) {
     }
   }
   __syncthreads();
+}
+
+// End of a CG update, by one thread after every block's work: |r|^2, the old rz of
+// the next direction, the count of updates, and |r|^2 and then the count to the
+// host's mapped slot.
+__device__ __forceinline__ void cg_publish(double* scal, double rr, double* host_rr) {
+  const double count = scal[S_CG_COUNT] + 1.0;
+  scal[S_RR] = rr;
+  scal[S_RZ0] = scal[S_RZ1];
+  scal[S_CG_COUNT] = count;
+  volatile double* h = host_rr;
+  h[0] = rr;
+  __threadfence_system();
+  h[1] = count;
+  __threadfence_system();
 }
 
 // Programmatic dependent launch.  A kernel launched by launch_pdl() may be
@@ -404,12 +420,15 @@ struct to_ctx {
   std::string last_error;
   long long launches;
   unsigned prof_mask;   // bit k: time launches of profiling kind k
-  // V-cycles captured as CUDA graphs, keyed by their buffers and precision
+  // V-cycles and whole CG iterations captured as CUDA graphs, keyed by their
+  // buffers (all in the workspace) and kind: the type of a V-cycle's result, or
+  // CG_ITERATION
+  static constexpr int CG_ITERATION = 100, MAX_VGRAPH = 8;
   struct VGraph {
     const void* rin;
     const void* zout;
     const void* coef;
-    int zt;
+    int kind;
     bool pre;   // right-hand side and pre-smoothing already in place
     cudaGraphExec_t exec;
     long long launches;
@@ -429,12 +448,11 @@ struct to_ctx {
   double oc_eta;          // damping exponent of the OC update
   int vf_l0;             // its first level (0: no level qualifies)
   float* tc_bmat;        // its B operand (device, 2 x 1024 floats)
-  VGraph vgraph[4];
+  VGraph vgraph[MAX_VGRAPH];
   int n_vgraph;
   cudaStream_t cap_stream;   // private stream used only for graph capture
   double* host_rr;           // pinned host slot for the CG residual read
   double* host_rr_dev;       // the same slot as the device addresses it (mapped)
-  cudaEvent_t rr_event;      // marks that read on the context stream
   std::vector<cudaEvent_t> ev_pool;
   std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev_used;
   std::vector<double> ev_bytes;
