@@ -119,11 +119,11 @@ to_status to_set_density(to_ctx* ctx, const double* rho_phys);
  *   the oldest column when full (Sec. 3.1).
  * iters (host, may be NULL): CG iterations taken; relres (host, may be
  *   NULL): final relative residual.  This call synchronises the stream.
- * The host reads |r|^2 once per CG iteration; the read is enqueued before
- * the next preconditioner application and waited on after it, so the
- * V-cycle runs during the round trip (its result is discarded on the
- * iteration that stops).  The first call on a context allocates 64 bytes of
- * pinned host memory for that read (released by to_destroy).
+ * The host reads |r|^2 once per CG iteration from pinned memory that the
+ * update kernel writes, while the next V-cycle runs (its result is discarded
+ * on the iteration that stops).  The first call on a context allocates 64
+ * bytes of that memory, and iterations in the middle of a solve replay as CUDA
+ * graphs captured when first needed (both released by to_destroy).
  * The first solve after to_set_density rebuilds the multigrid hierarchy; in
  * TO_MIXED the coarsest matrix's explicit inverse is formed in float32 and
  * checked (one small synchronising read), and a context whose float32
@@ -174,14 +174,15 @@ to_status to_carm_build(to_ctx* ctx, const double* u_last);
  *     solver (float32 in TO_MIXED, float64 in TO_FP64) as K p, as the
  *     V-cycle's residual and as its post-smoother;
  *   TO_TUNE_GAL1_RESID / _SMOOTH: the level-1 Galerkin operator applied
- *     from the finest moduli (3D, >= 3 levels);
+ *     from the finest moduli (3D, >= 3 levels; the solver uses it in
+ *     TO_MIXED, TO_FP64 stores that level);
  *   TO_TUNE_ACC_APPLY / _RESID: the double-float operator (TO_MIXED).
  * For the float32 finest-grid kernels it also times the 16-row tile
  * variant (TO_OPERATOR_TALL_TILES) and the work-list launch of either tile
  * (TO_OPERATOR_WORK_LIST).
  * It keeps the fastest (the occupancy heuristic's own shape when within 1 %
  * of it), applies it to every later launch of that kernel on this context,
- * drops the captured V-cycle graphs so that they are recaptured with it, and
+ * drops the captured graphs so that they are recaptured with it, and
  * caches it for the process under (device, kernel, grid), so later
  * contexts of the same grid take it without timing.  Results do not depend
  * on the chunking (every node sums its element contributions in the same
@@ -359,7 +360,7 @@ to_status to_filter(to_ctx* ctx, int32_t mode, const double* in, double* out);
 
 /* Optimality-criteria update of the design rho (dev, float64, nel, in/out):
  * rho_new = clamp(rho sqrt(max(0, -dc_f/(lam dv_f))), max(0, rho-move),
- * min(1, rho+move)) with lam chosen by bisection on [0, 1e9] to a relative
+ * min(1, rho+move)) with lam searched on [0, 1e9] to a relative
  * bracket of 1e-13 so that sum_e dv_f,e rho_new,e = volfrac*nel (the
  * filtered volume when dv_f = H^T(1/Hs), Eq. 3).  dc_f, dv_f: dev nel.
  * change_dev (dev, 1 double, may be NULL): max |rho_new - rho|. */
@@ -393,7 +394,8 @@ to_status to_oc_update_noalloc(int64_t nel, double volfrac, double move, const d
 /* y = op(x) for x, y dev float64 n (no aliasing).  op: TO_OP_K (current
  * stiffness with BCs, Eq. 7), TO_OP_KREF (reference stiffness, Eq. 8) or
  * TO_OP_DK (dK = K - K_ref, zero on fixed DOFs).  prec: TO_PREC_NATIVE
- * (the context's apply precision), TO_PREC_FP64, TO_PREC_FP32 (3D: x is
+ * (the context's apply precision), TO_PREC_FP64 (3D: products in 64-bit fixed
+ * point, no further from the exact result than float64's), TO_PREC_FP32 (3D: x is
  * rounded to float32 and the float32-storage operator of the mixed solver
  * runs; y is its result widened) or
  * TO_PREC_DF (3D: double-float arithmetic on the FP32 pipe, ~2^-48
@@ -402,7 +404,8 @@ to_status to_oc_update_noalloc(int64_t nel, double volfrac, double move, const d
 to_status to_apply(to_ctx* ctx, int32_t op, int32_t prec, const double* x, double* y);
 
 /* One V-cycle of the current hierarchy (Algorithm 2): z ~= K^{-1} r, with
- * r, z dev float64 n (builds the hierarchy if stale). */
+ * r, z dev float64 n, r != z (builds the hierarchy if stale).  r may be nonzero
+ * on fixed DOFs, where the operator is the identity. */
 to_status to_vcycle(to_ctx* ctx, const double* r, double* z);
 
 /* Galerkin operator of level l >= 1 (coarse grid l of the hierarchy):
