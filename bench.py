@@ -349,7 +349,7 @@ def run_ours(args):
              "k_apply3_pair<EPI_APPLY> (finest-grid K p, float32, two element columns per thread)")
     if n_f == 0:   # float64 path: the finest-grid operator runs in float64
         n_f, ms_f, by_f = n_o, ms_o, by_o
-        kname = "k_apply3_col<double> (finest-grid K p, float64)"
+        kname = "k_apply3_fx (finest-grid K p, float64 in 64-bit fixed point)"
 
     # ---- the same workload in plain float64 (the comparison the target names) ----
     fp64 = None
@@ -582,7 +582,7 @@ def run_kernel_apply(args):
     n, ms, by = B.to_profile_read(s.ctx, kind)
     s.close()
     return {"kernel": ("k_apply3_tc" if args.tensor_cores else "k_apply3_pair")
-            if args.kernel_prec == "fp32" else "k_apply3_col<double>",
+            if args.kernel_prec == "fp32" else "k_apply3_fx",
             "precision": args.kernel_prec,
             "launches": n,
             "avg_us": ms / n * 1e3, "GB/s": by / (ms / 1e3) / 1e9,
