@@ -196,15 +196,14 @@ __device__ __forceinline__ void wht4_dfl(dfl (&v)[4]) {
 // above (one element per thread read, split and transformed 24: 334 us at
 // 192 x 96 x 96, now 158), and the quadratic form takes the 33 non-zero entries of the
 // blocks' upper triangles instead of all 72.
-constexpr int SNX = 32, SNY = 4;
-__global__ void __launch_bounds__(SNX * SNY, 6)
+__global__ void __launch_bounds__(SN_X * SN_Y, 6)
     k_sensitivity3_df(GridP g, const uint8_t* __restrict__ mask, WhtDf kb, int zc,
                       const double* __restrict__ u, const double* __restrict__ E,
                       const double* __restrict__ rho, double pfac, int ipen,
                       double* __restrict__ dc, double* compliance, double* partials,
                       unsigned* counter) {
-  __shared__ double sh[1][SNX * SNY / 32], tot[1];
-  const int ex = blockIdx.x * SNX + threadIdx.x % SNX, ey = blockIdx.y * SNY + threadIdx.x / SNX;
+  __shared__ double sh[1][SN_X * SN_Y / 32], tot[1];
+  const int ex = blockIdx.x * SN_X + threadIdx.x % SN_X, ey = blockIdx.y * SN_Y + threadIdx.x / SN_X;
   const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, g.nz);
   const long long plane = (long long)g.nnx * g.nny;
   const dfl pf = split_d(pfac);
@@ -697,14 +696,11 @@ cudaError_t launch_sensitivity_df(const GridP& g, const uint8_t* mask, const dou
     (&kb.h[0][0][0])[q] = h;
     (&kb.l[0][0][0])[q] = (float)(w - (double)h);
   }
-  const int gx = (g.nx + SNX - 1) / SNX, gy = (g.ny + SNY - 1) / SNY;
-  // z-chunk: its first face is loaded and transformed again, so as long as the
-  // blocks still fill the SMs (six resident on each)
-  int zc = 16;
-  while (zc > 1 && (long long)gx * gy * ((g.nz + zc - 1) / zc) < 6 * 152) zc /= 2;
-  k_sensitivity3_df<<<dim3(gx, gy, (g.nz + zc - 1) / zc), SNX * SNY, 0, s>>>(
-      g, mask, kb, zc, u, E, rho, -penal * (E0 - Emin), (int)penal - 1, dc, compliance, partials,
-      counter);
+  const int zc = sensitivity_chunk(g.nx, g.ny, g.nz);
+  if (sensitivity_blocks(g.nx, g.ny, g.nz, zc) > PARTIALS) return cudaErrorInvalidValue;
+  const dim3 grid((g.nx + SN_X - 1) / SN_X, (g.ny + SN_Y - 1) / SN_Y, (g.nz + zc - 1) / zc);
+  k_sensitivity3_df<<<grid, SN_X * SN_Y, 0, s>>>(g, mask, kb, zc, u, E, rho, -penal * (E0 - Emin),
+                                                (int)penal - 1, dc, compliance, partials, counter);
   return cudaGetLastError();
 }
 

@@ -345,7 +345,7 @@ static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
   const bool l1_implicit = l2_tables && !store_level1(d);
   double* R2_64 = l2_tables ? cv.take<double>((size_t)64 * 576) : nullptr;
   float* R2_32 = l2_tables ? cv.take<float>((size_t)64 * 576) : nullptr;
-  double* partials = cv.take<double>((size_t)RED_BLOCKS * MAXB * MAXB);
+  double* partials = cv.take<double>((size_t)PARTIALS);
   unsigned* counters = cv.take<unsigned>(C_NCOUNTERS);
   double* scal = cv.take<double>(S_NSLOTS);
   double* small = cv.take<double>(SM_TOTAL);

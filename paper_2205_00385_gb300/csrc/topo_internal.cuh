@@ -9,12 +9,11 @@
 #include <vector>
 
 #include "../../include/topo.h"
+#include "launch_shapes.h"
 
 namespace topo {
 
 constexpr int MAXL = 10;        // multigrid levels
-constexpr int MAXB = 16;        // PARM / CARM columns
-constexpr int RED_BLOCKS = 608; // fixed grid of deterministic reductions (4 x 152 SMs)
 constexpr int RED_THREADS = 256;
 constexpr int MAX_STENCIL = 128;
 
