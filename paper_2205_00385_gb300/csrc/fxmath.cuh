@@ -32,13 +32,6 @@ typedef long long fx_t;
 constexpr int FX_S = 5, FX_C = 60;
 static_assert(FX_S + FX_C <= 66, "three products of high and low halves fit 63 bits");
 
-// the Walsh blocks in fixed point: entry = (hi 2^32 + lo) 2^(bs - 60), both
-// halves signed
-struct FxBlocks {
-  int hi[8][3][3], lo[8][3][3];
-  int bs;
-};
-
 struct FxFace {
   fx_t w[3][4];   // xy-Walsh sums of the face's four nodes per component
   int e;          // largest exponent field of the values

@@ -141,7 +141,7 @@ cudaError_t run_fx(const ApplyArgs& a, cudaStream_t s) {
   }
   if (a.zsplit > 0) zc = min(a.zsplit, (int)a.g.nnz);   // chosen by the autotuner
   return launch_pdl(k_apply3_fx<EPI>, dim3(gx, gy, (a.g.nnz + zc - 1) / zc), dim3(FX_X * FX_Y), 0,
-                    s, a.g, a.mask, fx_blocks(static_cast<const double*>(a.wht)),
+                    s, a.g, a.mask, *a.fx,
                     static_cast<const double*>(a.coef), zc, static_cast<const double*>(a.x),
                     static_cast<double*>(a.y), static_cast<const double*>(a.b),
                     static_cast<const double*>(a.dinv), a.omega, a.dfix, a.clean_inputs);
@@ -155,8 +155,10 @@ void fx_prepare() {
   fx_slots<EPI_SMOOTH>();
 }
 
+FxBlocks make_fx_blocks(const double* wht64) { return fx_blocks(wht64); }
+
 bool fx_apply_ok(const ApplyArgs& a) {
-  return a.dim == 3 && !a.expl && !a.gal1 && a.wht != nullptr && a.tc == T_F64 &&
+  return a.dim == 3 && !a.expl && !a.gal1 && a.fx != nullptr && a.tc == T_F64 &&
          a.tx == T_F64 && a.ty == T_F64;
 }
 

@@ -75,6 +75,13 @@ struct WhtBlocks {
   TC b[8][3][3];
 };
 
+// The Walsh blocks in fixed point (fxmath.cuh): entry = (hi 2^32 + lo)
+// 2^(bs - 60), both halves signed
+struct FxBlocks {
+  int hi[8][3][3], lo[8][3][3];
+  int bs;
+};
+
 // Structural zeros of the Walsh blocks of an isotropic hex8 KE: for a
 // single-bit character tau = e_k the translation component k decouples
 // (row and column zero); for a two-bit character the third component
@@ -415,6 +422,7 @@ struct to_ctx {
   float KE32[576];
   double wht64[72];   // Walsh-Hadamard blocks of KE (3D only)
   float wht32[72];
+  topo::FxBlocks fx;  // and in fixed point (1.6 us of host work to form)
   topo::StencilP stencil;
   std::string last_error;
   long long launches;
