@@ -394,8 +394,10 @@ to_status to_oc_update_noalloc(int64_t nel, double volfrac, double move, const d
 /* y = op(x) for x, y dev float64 n (no aliasing).  op: TO_OP_K (current
  * stiffness with BCs, Eq. 7), TO_OP_KREF (reference stiffness, Eq. 8) or
  * TO_OP_DK (dK = K - K_ref, zero on fixed DOFs).  prec: TO_PREC_NATIVE
- * (the context's apply precision), TO_PREC_FP64 (3D: products in 64-bit fixed
- * point, no further from the exact result than float64's), TO_PREC_FP32 (3D: x is
+ * (the context's apply precision), TO_PREC_FP64 (3D with nu < 0.37: an element's
+ * forces in 64-bit fixed point, off by a few units of 2^-61 of its largest strain
+ * mode times the largest entry of KE in norm, which is no more than float64
+ * arithmetic's rounding; otherwise float64), TO_PREC_FP32 (3D: x is
  * rounded to float32 and the float32-storage operator of the mixed solver
  * runs; y is its result widened) or
  * TO_PREC_DF (3D: double-float arithmetic on the FP32 pipe, ~2^-48

@@ -3,20 +3,28 @@
 // GB300 runs one float64 FMA per clock per SM, and integer adds and 32 x 32
 // -> 64 bit multiply-adds at tens per clock, so the ~230 additions and
 // multiplications of an element (corner Walsh-Hadamard basis, KE = T B T) run
-// on integers scaled to the element's own largest nodal value:
-//   value    v = u 2^(1075 + FX_S - e), e the largest exponent field among
-//            the four nodes of the face, truncated below 2^-57 of that value
+// on integers:
+//   values   each component of a face with the exponent of its own largest
+//            nodal value, FX_S bits below that value's mantissa kept
+//   modes    the 21 Walsh sums that strain the element (the three translations
+//            have no force and are left out), all scaled by one power of two
+//            so that the largest has FX_G bits
 //   moduli   60-bit mantissa with its own exponent
 //   B        entries scaled by 2^(60 - bs)
-// Additions are exact; a product drops its low 64 bits (4 units at most).  A
-// unit is 2^-57 of the largest nodal value, below float64's rounding of the
-// same sums (2^-53 of partial sums up to 8 times that value): over random,
-// smooth and mixed-scale elements at nu = 0.3 the rms error is 0.25 to 0.4 of
-// the float64 transform's.  Magnitudes: |v| < 2^58, Walsh sums < 2^61, and bs
-// is chosen on the host so that no intermediate of the inverse transform
-// reaches 2^62.  Results are
-// rounded once to float64.  Zeros are exact; an infinity or NaN among an
-// element's inputs makes all its outputs NaN.
+// Additions are exact; a product drops its low 64 bits (4 units at most).  So an
+// element's forces are off by a few units of 2^-FX_G of its largest strain mode
+// times the largest entry of B, in norm: a translation, or one component much
+// larger than the others, costs no bits.  (A component that the large modes
+// do not load, as u_z in a pure xy shear, has that same absolute error, where
+// float64 would round it at its own size.)  The float64 transform rounds every
+// sum at 2^-53 of the sum, translations included.  Measured against 80-bit
+// arithmetic at nu = 0.3, rms over elements, this / float64: random 0.37, linear
+// 0.12, quadratic 0.15, rigid rotation 0.05, one component uniform and the others
+// 1e-8 of it 0.38, magnitudes over 12 decades 0.37; about the same from nu = -0.95
+// to 0.35.  Towards 0.5 the entries of B spread (bulk to shear modulus) and one
+// unit no longer suits them all, see
+// fx_blocks_ok.  Results are rounded once to float64.  Zeros are exact; an
+// infinity or NaN among an element's inputs makes all its outputs NaN.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -28,13 +36,26 @@ namespace topo {
 
 typedef long long fx_t;
 
-// bits kept below a float64 mantissa's last, and bits of the constants
-constexpr int FX_S = 5, FX_C = 60;
-static_assert(FX_S + FX_C <= 66, "three products of high and low halves fit 63 bits");
+// Bits kept below a float64 mantissa's last, of the constants, and of the
+// largest strain mode.  A face's Walsh sums take 53 + FX_S + 2 bits, an element's
+// one more; products of halves: 3 (2^(FX_G - 1) + 2^59) < 2^63.  FX_S may be up to 7;
+// the errors above are the same with 5 and with 7 (0.01 of a ratio), and with 5 the
+// 48 x 24 x 24 design loop takes the oracle's CG iteration counts, which rounding
+// alone moves by a few on its gray designs.
+constexpr int FX_S = 5, FX_C = 60, FX_G = 61;
+static_assert(53 + FX_S + 3 <= 63 && FX_C <= 60 && FX_G <= 61, "sums and products fit 63 bits");
+
+__host__ __device__ __forceinline__ int fx_clz(unsigned long long m) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)m);
+#else
+  return m ? __builtin_clzll(m) : 64;
+#endif
+}
 
 struct FxFace {
   fx_t w[3][4];   // xy-Walsh sums of the face's four nodes per component
-  int e;          // largest exponent field of the values
+  int e[3];       // largest exponent field of the component's values
   bool bad;       // a value is not finite
 };
 
@@ -70,19 +91,17 @@ __host__ __device__ __forceinline__ void fx_wht4(fx_t (&v)[4]) {
 }
 
 __host__ __device__ __forceinline__ void fx_face(const double (&f)[4][3], FxFace& o) {
-  unsigned m = 0u;
+  o.bad = false;
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int c = 0; c < 3; ++c) {
+    unsigned m = 1u << 20;   // subnormal numbers have exponent field 1 too
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int q = 0; q < 4; ++q) {
       const unsigned h = (unsigned)(fx_bits(f[q][c]) >> 32) & 0x7fffffffu;
       m = h > m ? h : m;
     }
-  o.bad = m >= 0x7ff00000u;
-  o.e = (int)(m >> 20);
-  if (o.e < 1) o.e = 1;   // subnormal numbers have exponent field 1 too
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
+    o.bad = o.bad || m >= 0x7ff00000u;
+    o.e[c] = (int)(m >> 20);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const unsigned long long u = fx_bits(f[q][c]);
@@ -90,7 +109,7 @@ __host__ __device__ __forceinline__ void fx_face(const double (&f)[4][3], FxFace
       const int ef = (int)((h >> 20) & 0x7ffu);
       unsigned long long t = u & 0xfffffffffffffULL;
       t |= ef ? 1ULL << 52 : 0ULL;
-      const int s = o.e - (ef ? ef : 1);
+      const int s = o.e[c] - (ef ? ef : 1);
       t = (t << FX_S) >> (s < 63 ? s : 63);
       o.w[c][q] = (h >> 31) ? -(fx_t)t : (fx_t)t;
     }
@@ -109,17 +128,31 @@ __host__ __device__ __forceinline__ void fx_split(fx_t x, int& hi, int& lo) {
 __host__ __device__ __forceinline__ void fx_element(const FxBlocks& kb, double coef,
                                                     const FxFace& fb, const FxFace& ft,
                                                     double (&ye)[8][3]) {
-  const int e = fb.e > ft.e ? fb.e : ft.e;
-  const int sb = e - fb.e, st = e - ft.e;
+  // modes, and the least exponent e at which they all stay within FX_G bits
   fx_t X[3][8];
+  int ec[3], e = -4096;
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
+  for (int c = 0; c < 3; ++c) {
+    ec[c] = fb.e[c] > ft.e[c] ? fb.e[c] : ft.e[c];
+    const int sb = ec[c] - fb.e[c], st = ec[c] - ft.e[c];
+    unsigned long long m = 0;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const fx_t a = fx_shr(fb.w[c][t], sb), b = fx_shr(ft.w[c][t], st);
       X[c][t] = a + b;
       X[c][t + 4] = a - b;
+      if (t) m |= (unsigned long long)(X[c][t] ^ (X[c][t] >> 63));
+      m |= (unsigned long long)(X[c][t + 4] ^ (X[c][t + 4] >> 63));
     }
+    const int need = ec[c] + (64 - FX_G) - fx_clz(m);
+    if (m && need > e) e = need;
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int s = ec[c] - e, l = s > 0 ? s : 0, r = s < 0 ? -s : 0;
+#pragma unroll
+    for (int t = 1; t < 8; ++t) X[c][t] = fx_shr((fx_t)((unsigned long long)X[c][t] << l), r);
+  }
   // modulus: 60-bit signed mantissa, exponent field ee
   const unsigned long long cu = fx_bits(coef);
   const int cf = (int)((cu >> 52) & 0x7ff), ee = cf ? cf : 1;
@@ -134,6 +167,7 @@ __host__ __device__ __forceinline__ void fx_element(const FxBlocks& kb, double c
     int zh[3], zl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
+      if (tau == (1 << c)) continue;   // a translation
       int xh, xl;
       fx_split(X[c][tau ^ (1 << c)], xh, xl);
       const fx_t H = (fx_t)xh * ch, M = (fx_t)xh * cl + (fx_t)xl * ch;
@@ -180,47 +214,41 @@ __host__ __device__ __forceinline__ void fx_element(const FxBlocks& kb, double c
   }
 }
 
+// Whether one unit suits all entries of B: the largest at most FX_SPREAD times
+// the least of the diagonal, which holds for nu < 0.37.  The kind of field that
+// bounds it is a nearly rigid shear, whose force is small against its modes: at
+// nu = 0.35 (spread 6.5) its error is 0.29 to 0.4 of float64's, at 0.4 (9) 0.97, at
+// 0.45 (17) 2.4 and at 0.499 (750) 74 times it.
+constexpr double FX_SPREAD = 7.0;
+inline bool fx_blocks_ok(const double* wht) {
+  double mx = 0.0, mn = 1e300;
+  for (int tau = 0; tau < 8; ++tau)
+    for (int c = 0; c < 3; ++c)
+      for (int cp = 0; cp < 3; ++cp) {
+        const double v = fabs(wht[(tau * 3 + c) * 3 + cp]);
+        mx = fmax(mx, v);
+        if (c == cp && !wht_zero(tau, c, c)) mn = fmin(mn, v);
+      }
+  return mx <= FX_SPREAD * mn;
+}
+
 // Fixed-point form of the Walsh blocks (host).  bs is the least exponent such
 // that every entry is below 2^bs and every intermediate of the inverse
-// transform, whose largest possible value over inputs |v| < 2^(53 + FX_S) is its
-// coefficients' absolute sum, stays below 2^62.
+// transform, at most 2^FX_G times a component's absolute sum of entries, stays
+// below 2^62.
 inline FxBlocks fx_blocks(const double* wht) {
   auto at = [&](int tau, int c, int cp) { return wht[(tau * 3 + c) * 3 + cp]; };
   double mx = 0.0, grow = 0.0;
   for (int q = 0; q < 72; ++q) mx = fmax(mx, fabs(wht[q]));
-  double Y[3][8][24];   // Y[c][t] as a combination of the 24 nodal values
-  for (int tau = 0; tau < 8; ++tau)
-    for (int c = 0; c < 3; ++c)
-      for (int a = 0; a < 8; ++a)
-        for (int cp = 0; cp < 3; ++cp) {
-          const int t = tau ^ (1 << cp);
-          Y[c][tau ^ (1 << c)][3 * a + cp] =
-              (__builtin_popcount(a & t) & 1 ? -1.0 : 1.0) * at(tau, c, cp);
-        }
-  auto l1 = [&](const double* r) {
-    double s = 0.0;
-    for (int q = 0; q < 24; ++q) s += fabs(r[q]);
-    grow = fmax(grow, s);
-  };
-  // the transform's stages in the kernel's order: z, then x, then y
-  for (int c = 0; c < 3; ++c)
-    for (int t = 0; t < 8; ++t) l1(Y[c][t]);
-  const int order[3] = {4, 1, 2};
-  for (int s = 0; s < 3; ++s)
-    for (int c = 0; c < 3; ++c)
-      for (int t = 0; t < 8; ++t)
-        if (!(t & order[s])) {
-          for (int q = 0; q < 24; ++q) {
-            const double u = Y[c][t][q], v = Y[c][t | order[s]][q];
-            Y[c][t][q] = u + v;
-            Y[c][t | order[s]][q] = u - v;
-          }
-          l1(Y[c][t]);
-          l1(Y[c][t | order[s]]);
-        }
+  for (int c = 0; c < 3; ++c) {
+    double g = 0.0;
+    for (int tau = 0; tau < 8; ++tau)
+      for (int cp = 0; cp < 3; ++cp) g += fabs(at(tau, c, cp));
+    grow = fmax(grow, g);
+  }
   FxBlocks kb;
   kb.bs = -60;
-  while (ldexp(1.0, kb.bs) <= mx || ldexp(1.0, 9 - FX_S + kb.bs) <= grow) ++kb.bs;
+  while (ldexp(1.0, kb.bs) <= mx || ldexp(1.0, 62 - FX_G + kb.bs) <= grow) ++kb.bs;
   for (int tau = 0; tau < 8; ++tau)
     for (int c = 0; c < 3; ++c)
       for (int cp = 0; cp < 3; ++cp)

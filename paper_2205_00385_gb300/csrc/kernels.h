@@ -33,7 +33,8 @@ struct ApplyArgs {
   const void* ke;      // host pointer to the ND*ND element matrix of type tc
   const void* wht;     // host pointer to the 8x3x3 Walsh-Hadamard blocks of KE
                        // (type tc; 3D finest grid only, else null)
-  const FxBlocks* fx = nullptr;   // host pointer to the same in fixed point (float64 only)
+  const FxBlocks* fx = nullptr;   // host pointer to the same in fixed point
+                                  // (float64, where the blocks suit it)
   bool gal1;           // 3D level 1 without stored matrices: coef holds the
   GridP gf;            // finest-grid moduli, gf the finest grid
   const void* x;
@@ -94,8 +95,9 @@ cudaError_t launch_vcycle_coarse(int dim, int t, int ta, const VFuseArgs& a, cud
 // Float32 3D finest-grid operator, two element columns per thread with packed
 // f32x2 arithmetic (kernels_pair.cu); pair_apply_ok tells whether it applies.
 // float64 finest-grid hex8 operator with the element arithmetic in 64-bit
-// fixed point (kernels_fx.cu); its tables of the Walsh blocks wht64
-FxBlocks make_fx_blocks(const double* wht64);
+// fixed point (kernels_fx.cu); its tables of the Walsh blocks wht64, false where
+// the blocks do not suit it (the float64 transform then runs, kernels_fe.cu)
+bool make_fx_blocks(const double* wht64, FxBlocks* out);
 bool fx_apply_ok(const ApplyArgs& a);
 cudaError_t launch_apply_fx(const ApplyArgs& a, cudaStream_t s);
 void fx_prepare();

@@ -629,10 +629,9 @@ static cudaError_t run_col_epi(const ApplyArgs& a, cudaStream_t s) {
 template <int OP>
 static cudaError_t run_col_types(const ApplyArgs& a, cudaStream_t s) {
   if (a.tc == T_F64) {
-    // (the finest float64 operator runs in fixed point, kernels_fx.cu)
-    if constexpr (OP == OPK_GAL1)
-      if (a.tx == T_F64 && a.ty == T_F64) return run_col_epi<double, double, double, OP>(a, s);
-    return cudaErrorInvalidValue;
+    // (the finest operator only where fixed point, kernels_fx.cu, does not suit)
+    if (a.tx != T_F64 || a.ty != T_F64) return cudaErrorInvalidValue;
+    return run_col_epi<double, double, double, OP>(a, s);
   }
   if (a.tx == T_F32 && a.ty == T_F32) return run_col_epi<float, float, float, OP>(a, s);
   if (OP == OPK_FINE) {

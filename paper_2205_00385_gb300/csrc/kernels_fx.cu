@@ -12,9 +12,11 @@
 //
 // Bound by instruction issue and the FP64 pipe together (at 96 x 48 x 48, two
 // blocks per SM: issue 41 %, FP64 47 %, ALU 38 %); three blocks per SM (168
-// registers, a few spills) gain 8 to 20 %, four nothing more.  K x with float64
-// arithmetic / now: 53 / 17.5 us at 48 x 24 x 24, 156 / 57 us at 96 x 48 x 48,
-// 1115 / 310 us at 192 x 96 x 96.
+// registers) gain 8 to 20 %, four nothing more.  K x with float64 arithmetic / in
+// fixed point: 53 / 18.4 us at 48 x 24 x 24, 156 / 60 us at 96 x 48 x 48, 1115 /
+// 328 us at 192 x 96 x 96.  (Of that 1.6, 4 and 17 us scale the components and the
+// strain modes; with one exponent for a whole face a component far smaller than
+// another lost its bits.)
 #include "fxmath.cuh"
 #include "kernels.h"
 
@@ -155,7 +157,10 @@ void fx_prepare() {
   fx_slots<EPI_SMOOTH>();
 }
 
-FxBlocks make_fx_blocks(const double* wht64) { return fx_blocks(wht64); }
+bool make_fx_blocks(const double* wht64, FxBlocks* out) {
+  *out = fx_blocks(wht64);
+  return fx_blocks_ok(wht64);
+}
 
 bool fx_apply_ok(const ApplyArgs& a) {
   return a.dim == 3 && !a.expl && !a.gal1 && a.fx != nullptr && a.tc == T_F64 &&

@@ -494,6 +494,7 @@ to_status to_mesh_init(const to_mesh_desc* desc, const uint8_t* fixed_mask, cons
   c->vcycle_bytes = 0.0;
   c->coarse_t = c->mixed ? T_F32 : T_F64;
   c->coarse_shift = 0.0;
+  c->fx_ok = false;
   for (int q = 0; q < 8; ++q) c->tuned_zc[q] = c->tuned_var[q] = 0;
   c->carm_flags = 0;
   c->use_tc = false;
@@ -519,7 +520,7 @@ to_status to_mesh_init(const to_mesh_desc* desc, const uint8_t* fixed_mask, cons
       return fail(nullptr, TO_E_INVALID, "element Walsh blocks lack their structural zeros");
     }
     wht_blocks_pin_zeros(c->wht64, c->wht32);
-    c->fx = make_fx_blocks(c->wht64);
+    c->fx_ok = make_fx_blocks(c->wht64, &c->fx);
   }
   c->df_ok = c->dim == 3;
   std::vector<double> Qc((size_t)c->npe * c->nd * c->nd);
@@ -690,7 +691,7 @@ static ApplyArgs fine_args(const to_ctx* c, int op, int tc, int tx, int ty, cons
   const bool wide = tc == T_F64 || tc == T_DF;
   a.ke = wide ? (const void*)c->KE64 : (const void*)c->KE32;
   a.wht = c->dim == 3 ? (wide ? (const void*)c->wht64 : (const void*)c->wht32) : nullptr;
-  a.fx = c->dim == 3 && tc == T_F64 ? &c->fx : nullptr;
+  a.fx = c->dim == 3 && tc == T_F64 && c->fx_ok ? &c->fx : nullptr;
   a.gal1 = false;
   a.gf = c->lv[0].g;
   a.S = nullptr;

@@ -423,6 +423,7 @@ struct to_ctx {
   double wht64[72];   // Walsh-Hadamard blocks of KE (3D only)
   float wht32[72];
   topo::FxBlocks fx;  // and in fixed point (1.6 us of host work to form)
+  bool fx_ok;         // which suits this Poisson ratio
   topo::StencilP stencil;
   std::string last_error;
   long long launches;
