@@ -199,18 +199,37 @@ __host__ __device__ __forceinline__ void fx_element(const FxBlocks& kb, double c
     fx_wht4(b);
     fx_wht4(t);
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      const fx_t v = a < 4 ? b[a & 3] : t[a & 3];
-      // v 2^k: one rounding, then the exponent field; below the normal range
-      // the result is 0, above it infinite
-      unsigned long long d = fx_bits((double)v);
-      const int f = (int)((d >> 52) & 0x7ff) + k;
-      d += (unsigned long long)(long long)k << 52;
-      if (v == 0 || f <= 0) d = 0;
-      if (v != 0 && f >= 0x7ff) d = 0x7ff0000000000000ULL | (v < 0 ? 1ULL << 63 : 0ULL);
-      if (bad) d = 0x7ff8000000000000ULL;
-      ye[a][c] = fx_double(d);
+    for (int q = 0; q < 4; ++q) {
+      X[c][q] = b[q];
+      X[c][q + 4] = t[q];
     }
+  }
+  if (k > -1023) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int a = 0; a < 8; ++a) {
+        // v 2^k: one rounding, then the exponent field; above the range infinite
+        const fx_t v = X[c][a];
+        unsigned long long d = fx_bits((double)v);
+        const int f = (int)((d >> 52) & 0x7ff) + k;
+        d += (unsigned long long)(long long)k << 52;
+        if (v == 0) d = 0;
+        if (v != 0 && f >= 0x7ff) d = 0x7ff0000000000000ULL | (v < 0 ? 1ULL << 63 : 0ULL);
+        if (bad) d = 0x7ff8000000000000ULL;
+        ye[a][c] = fx_double(d);
+      }
+  } else {
+    // results may lie below the normal range: 2^k as two factors (v 2^(k / 2) is
+    // normal and exact, so the second product rounds as the number system does)
+    const int kk = k > -1200 ? k : -1200, k1 = kk / 2;
+    const double f1 = fx_double((unsigned long long)(1023 + k1) << 52);
+    const double f2 = fx_double((unsigned long long)(1023 + kk - k1) << 52);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+        ye[a][c] = bad ? fx_double(0x7ff8000000000000ULL) : (double)X[c][a] * f1 * f2;
   }
 }
 

@@ -13,8 +13,8 @@
 // Bound by instruction issue and the FP64 pipe together (at 96 x 48 x 48, two
 // blocks per SM: issue 41 %, FP64 47 %, ALU 38 %); three blocks per SM (168
 // registers) gain 8 to 20 %, four nothing more.  K x with float64 arithmetic / in
-// fixed point: 53 / 18.4 us at 48 x 24 x 24, 156 / 60 us at 96 x 48 x 48, 1115 /
-// 328 us at 192 x 96 x 96.  (Of that 1.6, 4 and 17 us scale the components and the
+// fixed point: 53 / 18.0 us at 48 x 24 x 24, 156 / 62 us at 96 x 48 x 48, 1115 /
+// 329 us at 192 x 96 x 96.  (Of that 1.3, 5 and 18 us scale the components and the
 // strain modes; with one exponent for a whole face a component far smaller than
 // another lost its bits.)
 #include "fxmath.cuh"

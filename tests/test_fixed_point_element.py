@@ -153,3 +153,23 @@ def test_poisson_ratios(lib, nu, ok):
     """Near 0.5 the entries of the Walsh blocks spread too far for one unit; the
     float64 transform runs there."""
     assert _blocks(lib, nu)[0] == ok
+
+
+def test_results_below_the_normal_range(lib):
+    """Subnormal results are rounded as the number system rounds them (1.5 units
+    of 2^-1074 with the product's own rounding), not flushed."""
+    ok, W = _blocks(lib, 0.3)
+    assert ok
+    rng = np.random.default_rng(18)
+    for scale in (1e-290, 1e-300, 1e-306, 1e-309, 1e-312, 1e-318, 1e-323):
+        for E in (1.0, 1e-9, 3e5, 1e-300):
+            u = rng.standard_normal(24) * scale
+            y, ref, e = np.zeros(24), np.zeros(24), np.zeros(2)
+            lib.fixed(_ptr(W), ctypes.c_double(E), _ptr(u), _ptr(y))
+            big = np.ascontiguousarray(u * 2.0 ** 500 * 2.0 ** 500)   # (exact)
+            lib.fixed(_ptr(W), ctypes.c_double(E), _ptr(big), _ptr(ref))
+            with np.errstate(under="ignore"):
+                ref = ref * 2.0 ** -500 * 2.0 ** -500
+            assert np.all(np.abs(y - ref) <= 1.5 * 2.0 ** -1074 + 1e-15 * np.max(np.abs(ref)))
+            if scale == 1e-309 and E == 1.0:
+                assert np.all(y != 0.0) and np.max(np.abs(y)) < 2.0 ** -1022

@@ -67,3 +67,22 @@ def test_vcycle(nu):
         z = dev(np.zeros(p.ndof))
         B.to_vcycle(c.ctx, dev(r), z)
         assert np.max(np.abs(host(z) - ref)) <= 1e-10 * np.max(np.abs(ref))
+
+
+def test_subnormal_results():
+    """Results below the normal range keep their bits.  Both sides round every
+    product or element force at 2^-1074: 128 units for the oracle's 81 per row."""
+    from paper_2205_00385_gb300 import binding as B
+    p = small_problem("cantilever3d", nelx=16, nely=8, nelz=8, mg_levels=2)
+    rho = rand_density(p.nel, 9, 0.1, 1.0)
+    E = sensitivity.simp_modulus(rho, p.E0, p.Emin, p.penal)
+    K = fe.stiffness(fe.Grid.of(p), E, fe.element_stiffness(3, p.nu), p.fixed)
+    x = 1e-312 * rand_vector(p.ndof, 10, fixed=p.fixed)
+    with Ctx(p, precision="fp64") as c:
+        c.set_density(rho)
+        y = dev(np.zeros(p.ndof))
+        B.to_apply(c.ctx, B.TO_OP_K, B.TO_PREC_FP64, dev(x), y)
+        y = host(y)
+    ref = K @ x
+    assert np.max(np.abs(ref)) > 1e-313
+    assert np.max(np.abs(y - ref)) <= 128 * 2.0 ** -1074
