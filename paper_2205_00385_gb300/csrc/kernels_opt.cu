@@ -615,7 +615,8 @@ __global__ void __launch_bounds__(RED_THREADS)
   __shared__ double sh[32];
   const double lam = 0.5 * (scal[S_OC_L1] + scal[S_OC_L2]);
   const double s = oc_lam_factor(lam, eta);
-  const long long inf = 0x7ff0000000000000LL, one = __double_as_longlong(1.0);
+  const long long inf = 0x7ff0000000000000LL, minus_inf = (long long)0xfff0000000000000ULL;
+  const long long one = __double_as_longlong(1.0);
   long long most = 0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nel;
        e += (long long)gridDim.x * blockDim.x) {
@@ -623,7 +624,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     long long lo = __double_as_longlong(r - move), hi = __double_as_longlong(r + move);
     long long t = __double_as_longlong(a[e] * s);
     lo = lo < 0 || lo > inf ? 0 : lo;
-    hi = hi > one ? one : hi;
+    hi = hi > one || (hi < 0 && hi > minus_inf) ? one : hi;   // (NaN of either sign: 1)
     t = t < lo || t > inf ? lo : t;
     t = t > hi ? hi : t;
     const double rn = __longlong_as_double(t);
