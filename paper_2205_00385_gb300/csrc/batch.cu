@@ -5,8 +5,8 @@
 // computes bitwise what it computes alone; the branches run concurrently on
 // the device and the host issues one launch per phase instead of one per
 // kernel per job.  Graphs are cached per job table and replayed while the
-// table (jobs, buffers, and the alternation of each job's two modulus
-// buffers, which both phases read) repeats, which it does every other
+// table (jobs, buffers, OC exponents, and the alternation of each job's two
+// modulus buffers, which both phases read) repeats, which it does every other
 // iteration of a steady set of jobs.
 #include <algorithm>
 #include <cstring>
@@ -109,8 +109,8 @@ extern "C" to_status to_batch_step(const to_batch_job* jobs, int32_t n, int32_t 
     seen.push_back(j.ctx);
   }
   cudaStream_t s = (cudaStream_t)stream;
-  // the job table (and, for the density phase, which modulus buffer each
-  // job writes next) identifies the graph
+  // the job table, each job's OC exponent and which modulus buffer it writes
+  // next identify the graph
   std::vector<uintptr_t> key{(uintptr_t)phase, (uintptr_t)n, (uintptr_t)s};
   for (int i = 0; i < n; ++i) {
     const to_batch_job& j = jobs[i];
@@ -124,6 +124,7 @@ extern "C" to_status to_batch_step(const to_batch_job* jobs, int32_t n, int32_t 
     key.push_back((uintptr_t)j.ctx->E64);
     key.push_back((uintptr_t)j.ctx->Eprev64);
     key.push_back((uintptr_t)j.ctx->have_density);
+    key.push_back(bits(j.ctx->oc_eta));   // (to_oc_options) an argument of the OC kernels
   }
   std::lock_guard<std::mutex> lock(g_mu);
   auto it = g_graphs.find(key);
