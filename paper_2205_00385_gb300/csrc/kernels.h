@@ -270,7 +270,8 @@ cudaError_t launch_cg_p_d2(long long n, void* p, float* p32, const float* z, con
 cudaError_t launch_small_spd_inverse(int m, const int* m_dev, const double* A, double* Ainv,
                                      int* status, cudaStream_t s);
 cudaError_t launch_small_matvec(int m, const int* m_dev, const double* A, const double* x,
-                                double* y, double sign, cudaStream_t s);
+                                double* y, double sign, cudaStream_t s,
+                                bool unit = false);
 cudaError_t launch_small_chol_solve(int m, const int* m_dev, const double* A, const double* b,
                                     double* x, int* status, cudaStream_t s);
 // truncated SVD of the unit-column basis from its QR factor (one warp):

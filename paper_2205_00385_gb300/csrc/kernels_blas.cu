@@ -201,14 +201,21 @@ __global__ void k_small_spd_inverse(int mmax, const int* m_dev, const double* A,
   (void)status;
 }
 
-// y = sign * A x (A column-major m x m), a row per lane
+// y = sign * A x (A column-major m x m), a row per lane; with unit set scaled by
+// the power of two that brings its largest entry into [1, 2)
 __global__ void k_small_matvec(int mmax, const int* m_dev, const double* A, const double* x,
-                               double* y, double sign) {
+                               double* y, double sign, bool unit) {
+  if (blockIdx.x != 0) return;
   const int m = m_dev ? min(*m_dev, mmax) : mmax, i = threadIdx.x;
-  if (i >= m || blockIdx.x != 0) return;
   double s = 0.0;
-  for (int k = 0; k < m; ++k) s += A[i + m * k] * x[k];
-  y[i] = sign * s;
+  if (i < m)
+    for (int k = 0; k < m; ++k) s += A[i + m * k] * x[k];
+  if (unit) {   // (exponent fields 1 .. 2045: numbers whose factor is normal too)
+    const unsigned hi = (unsigned)__double2hiint(s) & 0x7fffffffu;
+    const unsigned ef = __reduce_max_sync(0xffffffffu, hi) >> 20;
+    if (ef >= 1 && ef <= 2045) s *= __hiloint2double((int)((2046u - ef) << 20), 0);
+  }
+  if (i < m) y[i] = sign * s;
 }
 
 __global__ void k_small_chol_solve(int mmax, const int* m_dev, const double* A, const double* b,
@@ -400,8 +407,8 @@ cudaError_t launch_small_spd_inverse(int m, const int* m_dev, const double* A, d
 }
 
 cudaError_t launch_small_matvec(int m, const int* m_dev, const double* A, const double* x,
-                                double* y, double sign, cudaStream_t s) {
-  k_small_matvec<<<1, 32, 0, s>>>(m, m_dev, A, x, y, sign);
+                                double* y, double sign, cudaStream_t s, bool unit) {
+  k_small_matvec<<<1, 32, 0, s>>>(m, m_dev, A, x, y, sign, unit);
   return cudaGetLastError();
 }
 

@@ -1463,6 +1463,10 @@ to_status to_carm_build(to_ctx* c, const double* u_last) {
                             c->counters + C_MULTI, s), "K_Phi");
   LAUNCH(c, launch_small_spd_inverse(Ns, nullptr, small + SM_KPHI, small + SM_KPHI_INV,
                                      c->ints + I_STATUS, s), "K_Phi inverse");
+  // A column's scale changes neither the basis nor the solution, so each
+  // column's coefficients are brought to order 1 by a power of two: with a small
+  // design change |C| is small too, and the pairs' float32 exponents end at
+  // 1e-38, which the squares of C^5 u reach at |C| = 1e-4.
   // r_1 = u_last (or Phi K_Phi^{-1} Phi^T f, the alternative of Fig. 2);
   // r_i = -Phi K_Phi^{-1} Phi^T dK r_{i-1}  (Eq. 18-20, 26)
   if (c->carm_flags & TO_CARM_R1_PROJECTED_LOAD) {
@@ -1470,7 +1474,7 @@ to_status to_carm_build(to_ctx* c, const double* u_last) {
     LAUNCH(c, launch_gram(n, v, c->Phi, Ns, nullptr, fv, 1, nullptr, small + SM_Z, Ns,
                           c->partials, c->counters + C_MULTI, s), "Phi^T f");
     LAUNCH(c, launch_small_matvec(Ns, nullptr, small + SM_KPHI_INV, small + SM_Z, small + SM_W,
-                                  1.0, s), "K_Phi^-1 Phi^T f");
+                                  1.0, s, true), "K_Phi^-1 Phi^T f");
     LAUNCH(c, launch_combine(n, v, c->Phi, Ns, nullptr, small + SM_W, 1.0, 0.0, c->R, v, nullptr,
                              nullptr, c->partials, c->counters + C_UPD, s), "r1");
   } else {
@@ -1483,7 +1487,7 @@ to_status to_carm_build(to_ctx* c, const double* u_last) {
     LAUNCH(c, launch_gram(n, v, c->Phi, Ns, nullptr, c->t, 1, nullptr, small + SM_Z, Ns,
                           c->partials, c->counters + C_MULTI, s), "Phi^T t");
     LAUNCH(c, launch_small_matvec(Ns, nullptr, small + SM_KPHI_INV, small + SM_Z, small + SM_W,
-                                  -1.0, s), "K_Phi^-1 z");
+                                  -1.0, s, true), "K_Phi^-1 z");
     LAUNCH(c, launch_combine(n, v, c->Phi, Ns, nullptr, small + SM_W, 1.0, 0.0,
                              c->R + (size_t)i * n, v, nullptr, nullptr, c->partials,
                              c->counters + C_UPD, s), "r_i");
