@@ -822,22 +822,21 @@ static void combine_t(long long n, const void* A, int m, const int* m_dev, const
                                                               ww, rr, partials, counter);
 }
 
+template <typename S>
+static cudaError_t combine_dots_t(long long n, const void* A, int m, const int* m_dev,
+                                  const double* c, void* y, double* h, double* partials,
+                                  unsigned* counter, cudaStream_t s) {
+  auto kern = m <= 4 ? k_combine_dots<S, 4> : m <= 12 ? k_combine_dots<S, 12> : k_combine_dots<S, MAXB>;
+  return launch_pdl(kern, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n, (const S*)A, m, m_dev, c, (S*)y,
+                    h, partials, counter);
+}
+
 cudaError_t launch_combine_dots(long long n, int vt, const void* A, int m, const int* m_dev,
                                 const double* c, void* y, double* h, double* partials,
                                 unsigned* counter, cudaStream_t s) {
-  if (m > 12 || m < 0) return cudaErrorInvalidValue;
-  if (vt == V_DF2) {
-    if (m <= 4)
-      return launch_pdl(k_combine_dots<float2, 4>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
-                        (const float2*)A, m, m_dev, c, (float2*)y, h, partials, counter);
-    return launch_pdl(k_combine_dots<float2, 12>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
-                      (const float2*)A, m, m_dev, c, (float2*)y, h, partials, counter);
-  }
-  if (m <= 4)
-    return launch_pdl(k_combine_dots<double, 4>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
-                      (const double*)A, m, m_dev, c, (double*)y, h, partials, counter);
-  return launch_pdl(k_combine_dots<double, 12>, dim3(vgrid(n)), dim3(RED_THREADS), 0, s, n,
-                    (const double*)A, m, m_dev, c, (double*)y, h, partials, counter);
+  if (m > MAXB || m < 0) return cudaErrorInvalidValue;
+  return vt == V_DF2 ? combine_dots_t<float2>(n, A, m, m_dev, c, y, h, partials, counter, s)
+                     : combine_dots_t<double>(n, A, m, m_dev, c, y, h, partials, counter, s);
 }
 
 cudaError_t launch_combine(long long n, int vt, const void* A, int m, const int* m_dev,
