@@ -17,7 +17,7 @@
 // launches cost more than the chain.  Launches overlap by programmatic
 // stream serialization.  Whole inverse, one block before / now: float64
 // n = 186 1.23 / 0.31 ms and n = 336 3.83 / 0.49 ms; float32 n = 336 0.71 /
-// 0.19 ms.
+// 0.21 ms.
 #include "kernels.h"
 
 namespace topo {
@@ -84,23 +84,39 @@ __device__ __forceinline__ bool factor_invert(T (&D)[NB][NB + 1], T (&X)[NB][NB 
   return ok;
 }
 
-// v - sum a_q b_q.  Large float32 matrices sum the products first, so that an
-// entry is rounded at its own magnitude once per panel and not NB times: at
-// n = 1386 (80 x 48 x 40 bridge) the mixed V-cycle is then 2.0e-7 from the float64
-// one and 1.6e-6 without.  At n = 336 there is nothing to gain (5.1e-7 and 5.3e-7 at
-// 192 x 96 x 96), and float64 has the bits to spare.
-constexpr int SUM_N = 512;
-template <int NB, typename T>
-__device__ __forceinline__ T take_products(T v, const T* a, const T* b, int n) {
-  if (sizeof(T) == 4 && n > SUM_N) {
-    T s = T(0);
-#pragma unroll
-    for (int q = 0; q < NB; ++q) s += a[q] * b[q];
-    return v - s;
+// Running sum of products.  In float32 it is compensated (products exact,
+// the additions' errors in a second word), so that an entry is rounded once per
+// panel: subtracting NB products one by one rounds it NB times, which a long
+// elimination adds up.  Error of the inverse in a two-level V-cycle, rms of 12
+// densities, one by one / compensated (LAPACK's float32 inverse): n = 336 1.8e-5 /
+// 5.4e-6 (4.8e-6), n = 480 3.7e-5 / 6.9e-6 (6.5e-6); n = 1188, products summed first /
+// compensated 1.6e-5 / 1.5e-5 (1.7e-5).  Whole inverse 0.19 -> 0.21 ms at n = 336.
+template <typename T>
+struct Sum {
+  T v = T(0);
+  __device__ __forceinline__ void add(T a, T b) { v += a * b; }
+  __device__ __forceinline__ T get() const { return v; }
+};
+template <>
+struct Sum<float> {
+  float v = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b), t = __fadd_rn(v, p), w = __fsub_rn(t, v);
+    const float e = __fadd_rn(__fsub_rn(v, __fsub_rn(t, w)), __fsub_rn(p, w));
+    lo = __fadd_rn(lo, __fadd_rn(e, __fmaf_rn(a, b, -p)));
+    v = t;
   }
+  __device__ __forceinline__ float get() const { return v + lo; }
+};
+
+// v - sum a_q b_q
+template <int NB, typename T>
+__device__ __forceinline__ T take_products(T v, const T* a, const T* b) {
+  Sum<T> s;
+  s.v = v;
 #pragma unroll
-  for (int q = 0; q < NB; ++q) v -= a[q] * b[q];
-  return v;
+  for (int q = 0; q < NB; ++q) s.add(-a[q], b[q]);
+  return s.get();
 }
 
 // Update with panel k (rows k0 .. k0 + NB), or, with k0 < 0, only the
@@ -129,7 +145,7 @@ __global__ void __launch_bounds__(CT * CT)
         const int i = a + ty, j = b + tx;
         // identity beyond n, so that the padding factors to itself
         T v = k1 + i < n && k1 + j < n ? W[(size_t)(k1 + i) * n + k1 + j] : T(i == j);
-        if (k0 >= 0) v = take_products<NB, T>(v, Ps[i], Ps[j], n);
+        if (k0 >= 0) v = take_products<NB>(v, Ps[i], Ps[j]);
         D[i][j] = v;
         if (a != b) D[j][i] = v;
       }
@@ -169,7 +185,7 @@ __global__ void __launch_bounds__(CT * CT)
       if (i < n && j < n) {
         // column block k of X starts here: what W holds there is A_ik
         const T v = schur || j0 < k0 ? W[(size_t)i * n + j] : T(0);
-        W[(size_t)i * n + j] = take_products<NB, T>(v, a[ty], b[tx], n);
+        W[(size_t)i * n + j] = take_products<NB>(v, a[ty], b[tx]);
       }
     }
   }
@@ -197,10 +213,10 @@ __global__ void __launch_bounds__(CT * CT)
 #pragma unroll
     for (int cb = 0; cb < NB; cb += CT) {
       const int c = cb + tx;
-      T v = T(0);
+      Sum<T> v;
 #pragma unroll
-      for (int q = 0; q < cb + CT; ++q) v += s[ty][q] * X[c][q];
-      if (i0 + ty < n) P[(size_t)(i0 + ty) * NB + c] = v;
+      for (int q = 0; q < cb + CT; ++q) v.add(s[ty][q], X[c][q]);
+      if (i0 + ty < n) P[(size_t)(i0 + ty) * NB + c] = v.get();
     }
   } else {
     const int j0 = CT * (b - nr);
@@ -213,10 +229,10 @@ __global__ void __launch_bounds__(CT * CT)
 #pragma unroll
       for (int rb = 0; rb < NB; rb += CT) {
         const int r = rb + ty;
-        T v = T(0);
+        Sum<T> v;
 #pragma unroll
-        for (int q = 0; q < rb + CT; ++q) v += X[r][q] * s[q][tx];
-        if (k0 + r < n) W[(size_t)(k0 + r) * n + j0 + tx] = v;
+        for (int q = 0; q < rb + CT; ++q) v.add(X[r][q], s[q][tx]);
+        if (k0 + r < n) W[(size_t)(k0 + r) * n + j0 + tx] = v.get();
       }
     } else {
       __syncthreads();
