@@ -324,7 +324,10 @@ cudaError_t launch_oc_prep_d(long long nel, const double* rho, const double* dc,
                              unsigned* counter, cudaStream_t s, double eta = 0.5);
 cudaError_t launch_oc_search(long long nel, const void* a2, const void* lo2, const void* hi2,
                              const void* dv2, double target, double* scal, double* partials,
-                             unsigned* counter, cudaStream_t s, double eta = 0.5);
+                             unsigned* counter, unsigned* turn, int* status, cudaStream_t s,
+                             double eta = 0.5);
+// caches the search's resident-block count for the current device
+void oc_prepare();
 cudaError_t launch_oc_final(long long nel, double* rho, const double* a, double move,
                             double* scal, double* change_dev, double* partials,
                             unsigned* counter, cudaStream_t s, double eta = 0.5);

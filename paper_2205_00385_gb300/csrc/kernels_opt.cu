@@ -425,14 +425,16 @@ __global__ void __launch_bounds__(RED_THREADS)
 //   lower end 0      l2 / 8^7 .. l2 / 8
 //   ratio above 4    geometric
 //   narrow           the secant point, +- guards of half the squared width and
-//                    1/32 of that, and the bracket's thirds, which bound the
-//                    sweeps when the secant point misses
-// Six or seven sweeps reach the relative bracket of 1e-13 (equal sections of
-// the bracket took 17 to 23); a sweep after that is a no-op, and one block
-// goes on where OC_SWEEPS were not enough, so that nothing waits for the host
-// and a captured update needs no more launches.  A sweep reads 32 bytes per
-// element (57 MB at 192 x 96 x 96, which stays in L2): 24 us there, of which the
-// arithmetic of the seven points is 8.
+//                    1/32 of that, and the bracket's thirds
+//   no slope (the volume changes by its own rounding), or the last narrow
+//   sweep left more than a fifth    equal sections
+// Six or seven sweeps reach the relative bracket of 1e-13 on most designs (equal
+// sections of the bracket took 17 to 23), up to 20 where the volume is nearly flat
+// in lambda.  A sweep after that is a no-op.  Where OC_SWEEPS were not enough one
+// launch goes on by itself (k_oc_rest), so that nothing waits for the host and a
+// captured update needs no more launches.  A sweep reads 32 bytes per element (57
+// MB at 192 x 96 x 96, which stays in L2): 24 us there, of which the arithmetic
+// of the seven points is 8.
 constexpr int OC_NP = 7, OC_T = 512, OC_BLOCKS = 304, OC_SWEEPS = 9;
 constexpr double OC_LAM_MAX = 1e9;
 static_assert(OC_NP <= S_OC_NPT && OC_NP <= OC_T / 32, "one warp per point");
@@ -456,10 +458,11 @@ __device__ __forceinline__ bool oc_done(double l1, double l2) {
 
 // Writes the bracket and its next points; called by one whole warp.
 // v1, v2 and s1, s2: the volumes and factors lambda^-eta at the bracket's ends
-// (of the lower end unknown, and not used, while it is 0).
+// (of the lower end unknown, and not used, while it is 0).  missed: the last
+// secant points did not narrow the bracket.
 __device__ __forceinline__ void oc_next_points(double l1, double l2, double v1, double v2,
                                                double s1, double s2, double target, double eta,
-                                               double l0, volatile double* scal) {
+                                               double l0, bool missed, volatile double* scal) {
   const int j = threadIdx.x & 31;
   double lam;
   if (l0 > 0.0) {
@@ -470,7 +473,7 @@ __device__ __forceinline__ void oc_next_points(double l1, double l2, double v1, 
     const double q = sqrt(sqrt(sqrt(l2 / l1)));
     lam = l1;
     for (int i = 0; i <= j && i < OC_NP; ++i) lam *= q;
-  } else if (!(v1 > v2)) {   // no slope: equal sections
+  } else if (missed || !(v1 - v2 > 1e-13 * target)) {
     lam = l1 + (j + 1) * ((l2 - l1) / (OC_NP + 1));
   } else {
     const double mid = oc_lam_of(s2 + (target - v2) * ((s1 - s2) / (v1 - v2)), eta);
@@ -545,62 +548,116 @@ __global__ void __launch_bounds__(OC_T)
   const double l2 = tot[1] > target ? OC_LAM_MAX : 0.0;
   const double st = oc_lam_factor(OC_LAM_MAX, eta);
   oc_next_points(l1, l2, tot[1], tot[2], st, st, target, eta,
-                 l0 > 1e-60 && l0 < OC_LAM_MAX ? l0 : 0.0, scal);
+                 l0 > 1e-60 && l0 < OC_LAM_MAX ? l0 : 0.0, false, scal);
 }
 
-// One sweep by the whole grid (LOOP: by one block, until the bracket is done;
-// a sweep at least thirds a bracket that does not start at 0 and takes one that
-// does down by 8^7, so the limit is not met).
-template <bool LOOP>
-__global__ void __launch_bounds__(OC_T, 2)
-    k_oc_sweep(long long nel, const float4* __restrict__ a, const float4* __restrict__ lo,
-               const float4* __restrict__ hi, const float4* __restrict__ dvd, double target,
-               volatile double* scal, double* partials, unsigned* counter, double eta) {
-  __shared__ double sh[OC_NP][OC_T / 32], tot[OC_NP];
-  pdl_wait();
-  for (int it = 0; it < (LOOP ? 160 : 1); ++it) {
-    const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
-    if (oc_done(l1, l2)) return;
-    dfl sv[OC_NP], v[OC_NP];
+struct OcFields {   // the elements' factors, limits and weights, two per float4
+  const float4 *a, *lo, *hi, *dv;
+};
+
+// The volumes at the sweep's points over the grid; true in the last block, where
+// tot holds them.
+template <typename Sh>
+__device__ __forceinline__ bool oc_volumes(long long nel, const OcFields& f, volatile double* scal,
+                                           Sh& sh, double (&tot)[OC_NP], double* partials,
+                                           unsigned* counter, bool trigger) {
+  dfl sv[OC_NP], v[OC_NP];
+#pragma unroll
+  for (int j = 0; j < OC_NP; ++j) {
+    sv[j] = split_d(scal[S_OC_SP + j]);
+    v[j] = {0.f, 0.f};
+  }
+  auto element = [&](dfl av, dfl lv, dfl hv, dfl dd) {
 #pragma unroll
     for (int j = 0; j < OC_NP; ++j) {
-      sv[j] = split_d(scal[S_OC_SP + j]);
-      v[j] = {0.f, 0.f};
+      dfl x = df_mul(av, sv[j]);
+      x = df_gt(x, hv) ? hv : (df_gt(lv, x) ? lv : x);
+      df_dot_acc(v[j], dd, x);
     }
-    auto element = [&](dfl av, dfl lv, dfl hv, dfl dd) {
+  };
+  // two elements per 16-byte load (nel is even: every grid coarsens once)
+  for (long long q = (long long)blockIdx.x * OC_T + threadIdx.x; 2 * q < nel;
+       q += (long long)gridDim.x * OC_T) {
+    const float4 a4 = __ldg(f.a + q), l4 = __ldg(f.lo + q), h4 = __ldg(f.hi + q), d4 = __ldg(f.dv + q);
+    element({a4.x, a4.y}, {l4.x, l4.y}, {h4.x, h4.y}, {d4.x, d4.y});
+    element({a4.z, a4.w}, {l4.z, l4.w}, {h4.z, h4.w}, {d4.z, d4.w});
+  }
 #pragma unroll
-      for (int j = 0; j < OC_NP; ++j) {
-        dfl x = df_mul(av, sv[j]);
-        x = df_gt(x, hv) ? hv : (df_gt(lv, x) ? lv : x);
-        df_dot_acc(v[j], dd, x);
+  for (int j = 0; j < OC_NP; ++j) v[j] = df_norm(v[j]);
+  if (trigger) pdl_launch_dependents();
+  return grid_sum_df(v, sh, tot, partials, counter);
+}
+
+// The sub-interval that holds the root, and its points; by one warp.  The volume
+// decreases with lambda: the last point above target and the first at or below it.
+__device__ __forceinline__ void oc_narrow(const double (&tot)[OC_NP], double target, double eta,
+                                          volatile double* scal) {
+  const double l1 = scal[S_OC_L1], l2 = scal[S_OC_L2];
+  int k = 0;
+  while (k < OC_NP && tot[k] > target) ++k;
+  const double n1 = k > 0 ? scal[S_OC_PT + k - 1] : l1;
+  const double w1 = k > 0 ? tot[k - 1] : scal[S_OC_V1];
+  const double f1 = scal[k > 0 ? S_OC_SP + k - 1 : S_OC_S1];
+  const double n2 = k < OC_NP ? scal[S_OC_PT + k] : l2;
+  const double w2 = k < OC_NP ? tot[k] : scal[S_OC_V2];
+  const double f2 = scal[k < OC_NP ? S_OC_SP + k : S_OC_S2];
+  const bool missed = l2 <= 4.0 * l1 && n2 - n1 > 0.2 * (l2 - l1);
+  __syncwarp();
+  oc_next_points(n1, n2, w1, w2, f1, f2, target, eta, 0.0, missed, scal);
+}
+
+// one sweep
+__global__ void __launch_bounds__(OC_T, 2)
+    k_oc_sweep(long long nel, OcFields f, double target, volatile double* scal, double* partials,
+               unsigned* counter, double eta) {
+  __shared__ double sh[OC_NP][OC_T / 32], tot[OC_NP];
+  pdl_wait();
+  if (oc_done(scal[S_OC_L1], scal[S_OC_L2])) return;
+  if (oc_volumes(nel, f, scal, sh, tot, partials, counter, true) && threadIdx.x < 32)
+    oc_narrow(tot, target, eta, scal);
+}
+
+// Sweeps until the bracket is done: blocks that are all resident (one cluster, or a
+// cooperative launch) wait for the last one's points, so the wait ends; its limit
+// of a few seconds sets *status.  A sweep at least thirds a bracket that does not start at
+// 0 and takes one that does down by 8^7, so the loop's limit is not met.
+constexpr int OC_WAIT = 1 << 22, OC_CLUSTER = 16;
+__global__ void __launch_bounds__(OC_T, 2)
+    k_oc_rest(long long nel, OcFields f, double target, volatile double* scal, double* partials,
+              unsigned* counter, volatile unsigned* turn, int* status, double eta) {
+  __shared__ double sh[OC_NP][OC_T / 32], tot[OC_NP];
+  __shared__ bool s_go;
+  pdl_wait();
+  unsigned t0 = 0;
+  if (threadIdx.x == 0) {
+    t0 = *turn;
+    __threadfence();   // (read before this block's first partial sums are counted)
+  }
+  for (int it = 0; it < 160; ++it) {
+    if (oc_done(scal[S_OC_L1], scal[S_OC_L2])) return;
+    const bool last = oc_volumes(nel, f, scal, sh, tot, partials, counter, false);
+    if (last && threadIdx.x < 32) oc_narrow(tot, target, eta, scal);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s_go = true;
+      if (last) {
+        __threadfence();
+        *turn = t0 + 1;
+      } else {
+        for (int w = 0; *turn == t0; ++w) {
+          if (w == OC_WAIT) {
+            *status = TO_E_TIMEOUT;
+            s_go = false;
+            break;
+          }
+          __nanosleep(40);
+        }
+        __threadfence();
       }
-    };
-    // two elements per 16-byte load (nel is even: every grid coarsens once)
-    for (long long q = (long long)blockIdx.x * OC_T + threadIdx.x; 2 * q < nel;
-         q += (long long)gridDim.x * OC_T) {
-      const float4 a4 = a[q], l4 = lo[q], h4 = hi[q], d4 = dvd[q];
-      element({a4.x, a4.y}, {l4.x, l4.y}, {h4.x, h4.y}, {d4.x, d4.y});
-      element({a4.z, a4.w}, {l4.z, l4.w}, {h4.z, h4.w}, {d4.z, d4.w});
+      ++t0;
     }
-#pragma unroll
-    for (int j = 0; j < OC_NP; ++j) v[j] = df_norm(v[j]);
-    if (!LOOP) pdl_launch_dependents();
-    if (!grid_sum_df(v, sh, tot, partials, counter)) return;
-    if (threadIdx.x < 32) {
-      // the volume decreases with lambda: keep the last point above target
-      // and the first at or below it
-      int k = 0;
-      while (k < OC_NP && tot[k] > target) ++k;
-      const double n1 = k > 0 ? scal[S_OC_PT + k - 1] : l1;
-      const double w1 = k > 0 ? tot[k - 1] : scal[S_OC_V1];
-      const double f1 = scal[k > 0 ? S_OC_SP + k - 1 : S_OC_S1];
-      const double n2 = k < OC_NP ? scal[S_OC_PT + k] : l2;
-      const double w2 = k < OC_NP ? tot[k] : scal[S_OC_V2];
-      const double f2 = scal[k < OC_NP ? S_OC_SP + k : S_OC_S2];
-      __syncwarp();
-      oc_next_points(n1, n2, w1, w2, f1, f2, target, eta, 0.0, scal);
-    }
-    if (LOOP) __syncthreads();
+    __syncthreads();
+    if (!s_go) return;
   }
 }
 
@@ -770,18 +827,76 @@ cudaError_t launch_oc_prep_d(long long nel, const double* rho, const double* dc,
   return cudaGetLastError();
 }
 
+// resident blocks of a cooperative k_oc_rest, and whether the device takes a
+// cluster of OC_CLUSTER (queried at set-up, outside any stream capture)
+struct OcShape {
+  int slots;
+  bool cluster;
+};
+static OcShape oc_shape() {
+  static OcShape cache[64] = {};
+  int dev = 0, sms = 0, per_sm = 0, clusters = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  if (cache[dev].slots > 0) return cache[dev];
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_oc_rest, OC_T, 0) != cudaSuccess ||
+      sms <= 0 || per_sm <= 0)
+    return {1, false};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(OC_CLUSTER);
+  cfg.blockDim = dim3(OC_T);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = OC_CLUSTER;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const bool ok =
+      cudaFuncSetAttribute(k_oc_rest, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&clusters, k_oc_rest, &cfg) == cudaSuccess && clusters > 0;
+  (void)cudaGetLastError();
+  return cache[dev] = {sms * per_sm, ok};
+}
+
+void oc_prepare() { oc_shape(); }
+
 cudaError_t launch_oc_search(long long nel, const void* a2, const void* lo2, const void* hi2,
                              const void* dv2, double target, double* scal, double* partials,
-                             unsigned* counter, cudaStream_t s, double eta) {
-  auto sweep = [&](auto kern, int blocks) {
-    return launch_pdl(kern, dim3(blocks), dim3(OC_T), 0, s, nel, (const float4*)a2,
-                      (const float4*)lo2, (const float4*)hi2, (const float4*)dv2, target, scal,
-                      partials, counter, eta);
-  };
+                             unsigned* counter, unsigned* turn, int* status, cudaStream_t s,
+                             double eta) {
+  const OcFields f = {(const float4*)a2, (const float4*)lo2, (const float4*)hi2, (const float4*)dv2};
+  const int blocks = oc_blocks(nel);
   cudaError_t e = cudaSuccess;
   for (int q = 0; q < OC_SWEEPS && e == cudaSuccess; ++q)
-    e = sweep(k_oc_sweep<false>, oc_blocks(nel));
-  return e == cudaSuccess ? sweep(k_oc_sweep<true>, 1) : e;
+    e = launch_pdl(k_oc_sweep, dim3(blocks), dim3(OC_T), 0, s, nel, f, target, scal, partials, counter,
+                   eta);
+  if (e != cudaSuccess) return e;
+  // The rest by one cluster up to 128 x 64 x 64 elements, else by the whole grid:
+  // cooperative launches in concurrent branches cost a batch of four served grids 20
+  // of 390 us.  Update with the target on a plateau of the volume, the rest by one
+  // block / so: 765 / 282 us at 48 x 24 x 24, 607 / 508 at 96 x 48 x 48 (430 by the
+  // whole grid), 39800 / 660 at 192 x 96 x 96, 217000 / 1910 at 320 x 160 x 160.
+  const OcShape sh = oc_shape();
+  const bool small = sh.cluster && nel <= 1 << 19;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(small ? OC_CLUSTER : std::min(blocks, sh.slots));
+  cfg.blockDim = dim3(OC_T);
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  cfg.attrs = at;
+  cfg.numAttrs = small ? 2 : 1;
+  if (small) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = OC_CLUSTER;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, k_oc_rest, nel, f, target, (volatile double*)scal, partials, counter,
+                            (volatile unsigned*)turn, status, eta);
 }
 
 cudaError_t launch_oc_final(long long nel, double* rho, const double* a, double move,

@@ -574,6 +574,7 @@ to_status to_mesh_init(const to_mesh_desc* desc, const uint8_t* fixed_mask, cons
                                                              c->lv[l].g, c->lv[l].mask);
     INIT_TRY(cudaGetLastError(), "coarse mask");
   }
+  oc_prepare();
   if (c->dim == 3) {
     pair_prepare();
     col_prepare();
@@ -1049,7 +1050,7 @@ static to_status check_status(to_ctx* c) {
   CUDA_TRY(c, cudaStreamSynchronize(c->stream), "sync");
   if (st[I_TIMEOUT]) {
     cudaMemsetAsync(c->ints + I_TIMEOUT, 0, 4, c->stream);
-    return fail(c, TO_E_TIMEOUT, "a bounded device wait expired (tensor-core operator)");
+    return fail(c, TO_E_TIMEOUT, "a bounded device wait expired (tensor-core operator or OC search)");
   }
   if (st[I_STATUS]) {
     cudaMemsetAsync(c->ints + I_STATUS, 0, 4, c->stream);
@@ -1867,7 +1868,8 @@ to_status oc_update_enqueue(to_ctx* c, double volfrac, double move, const double
                              c->oc_hi, c->oc_dv2, c->scal, c->partials, c->counters + C_OC, s,
                              c->oc_eta), "oc prep");
   LAUNCH(c, launch_oc_search(nel, c->oc_a2, c->oc_lo, c->oc_hi, c->oc_dv2, target, c->scal,
-                             c->partials, c->counters + C_OC, s, c->oc_eta), "oc search");
+                             c->partials, c->counters + C_OC, c->counters + C_OC_TURN,
+                             c->ints + I_TIMEOUT, s, c->oc_eta), "oc search");
   LAUNCH(c, launch_oc_final(nel, rho, c->oc_a, move, c->scal, change_dev, c->partials,
                             c->counters + C_MAX, s, c->oc_eta), "oc final");
   return TO_OK;

@@ -476,8 +476,9 @@ namespace topo {
 
 // Counter slots (ctx->counters, one per reduction site in flight)
 // C_PAIR: the float32 pair kernel's work-list counters, two per epilogue
+// C_OC_TURN: sweeps of the OC search's cooperative launch (never reset)
 enum Counter { C_DOT = 0, C_MULTI = 1 /* .. +16 */, C_UPD = 20, C_OC = 21, C_SENS = 22,
-               C_MAX = 23, C_PAIR = 24 /* .. +6 */, C_NCOUNTERS = 32 };
+               C_MAX = 23, C_PAIR = 24 /* .. +6 */, C_OC_TURN = 30, C_NCOUNTERS = 32 };
 
 // --- launch helpers (host) ---
 void note_launch(to_ctx* c);
