@@ -81,7 +81,11 @@ typedef struct to_mesh_desc {
   int32_t n_parm, n_carm;
 } to_mesh_desc;
 
-/* Bytes of device workspace needed for a problem (host-only query). */
+/* Bytes of device workspace needed for a problem (host-only query).  3D, one
+ * PARM and CARM column: about 500 bytes an element in TO_MIXED, 600 in TO_FP64, and
+ * 16 n for each further column; TO_FP64 with three grids or more also keeps
+ * its first coarse level's matrices, 565 bytes an element, where they are at most
+ * 8 GB in all. */
 to_status to_workspace_bytes(const to_mesh_desc* desc, int64_t* bytes);
 
 /* Create a solver context.

@@ -303,15 +303,18 @@ struct Carver {
 // 243 FMAs and 84 x 3 values per node.  In float64 (one FMA per clock per SM)
 // the FP64 pipe bounds the implicit form at every size: a V-cycle takes 466 us
 // with it and 171 us with the stencil at 48 x 24 x 24, 2267 and 1291 us at
-// 128 x 64 x 64.  It stays only beyond 8 GB, where the stencil and the element
-// matrices it is assembled from would crowd out the rest of the workspace.
+// 128 x 64 x 64.  Stencil and the element matrices it is assembled from take 565
+// bytes per finest element, about what the rest of the workspace does (1.0 GB of
+// 2.2 at 192 x 96 x 96, 4.6 of 9.6 at 320 x 160 x 160, one PARM and CARM column), so
+// the implicit form stays where they would be more than 8 GB (14 million elements).
 // In float32 level 1 is always implicit: the stencil gains 10 us of 90 at
 // 96 x 48 x 48 and loses from 128 x 64 x 64 on, and its rounded rows no longer
 // annihilate rigid motions, which costs iterations on designs with solid
 // parts hanging in near-void.
 static bool store_level1(const to_mesh_desc& d) {
+  const GridP g = level_grid(d, 1);
   return d.precision == TO_FP64 &&
-         8.0 * (double)stencil_values(3, T_F64, level_grid(d, 1)) <= 8e9;
+         8.0 * ((double)stencil_values(3, T_F64, g) + (double)tri_len(24) * g.nel) <= 8e9;
 }
 
 static size_t carve(const to_mesh_desc& d, to_ctx* c, char* base) {
