@@ -8,8 +8,9 @@ R the CARM basis (n x N_m).
 Readings of what the paper leaves open:
 * Eq. 16-17 are not valid for a non-square Phi; the approximate inverse is
   taken as the result they arrive at, Eq. 18: Phi (Phi^T K_ref Phi)^{-1} Phi^T.
-* K_Phi is inverted by Cholesky; if that fails, by the symmetric
-  eigen-pseudo-inverse with relative cutoff 1e-14.
+* K_Phi is inverted by Cholesky; if that fails, or leaves a pivot no larger
+  than the rounding of the sums it comes from (m units of its diagonal entry), by
+  the symmetric eigen-pseudo-inverse with relative cutoff 1e-14.
 * Eq. 21 (PCA by SVD) gives no truncation rule: the columns of R are first
   scaled to unit length (the span, and hence the reduced solution, does not
   depend on column scaling) and singular directions with
@@ -70,6 +71,9 @@ def small_spd_inverse(A: np.ndarray) -> np.ndarray:
     A = 0.5 * (A + A.T)
     try:
         c = sla.cho_factor(A)
+        pivots = np.diag(c[0]) ** 2
+        if np.any(pivots <= A.shape[0] * np.finfo(float).eps * np.diag(A)):
+            raise np.linalg.LinAlgError("singular to rounding")
         return sla.cho_solve(c, np.eye(A.shape[0]))
     except np.linalg.LinAlgError:
         w, V = np.linalg.eigh(A)
