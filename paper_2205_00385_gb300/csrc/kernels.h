@@ -150,10 +150,10 @@ cudaError_t launch_presmooth(int t, int tin, long long n, const void* bin, void*
                              const void* dinv, double omega, void* z, cudaStream_t s, int dim = 0,
                              const uint8_t* mask = nullptr);
 // float64 result of a V-cycle on an input r that may be nonzero on fixed DOFs:
-// out = zin (type t; null: out holds it already) on free DOFs, the operator
-// being the identity on fixed ones
-cudaError_t launch_vcycle_out(int dim, int t, long long n, const void* zin, const double* r,
-                              double omega, const uint8_t* mask, double* out, cudaStream_t s);
+// out = zin (the float32 cycle's result; null: out holds the float64 cycle's
+// already) on free DOFs, the operator being the identity on fixed ones
+cudaError_t launch_vcycle_out(int dim, long long n, const float* zin, const double* r, double omega,
+                              const uint8_t* mask, double* out, cudaStream_t s);
 cudaError_t launch_galerkin_fine(int dim, int t, const GridP& gc, const GridP& gf,
                                  const void* coef, const void* Qc, void* Kc, cudaStream_t s);
 cudaError_t launch_galerkin_coarse(int dim, int t, const GridP& gc, const GridP& gf,

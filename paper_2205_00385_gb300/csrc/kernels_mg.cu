@@ -135,15 +135,15 @@ __global__ void __launch_bounds__(EW_T)
   pdl_launch_dependents();
 }
 
-// Result of a V-cycle in float64: on a fixed DOF, where the operator is the
+// Float64 result of a float32 V-cycle: on a fixed DOF, where the operator is the
 // identity, two smoothing steps of the input; elsewhere zin.
-template <int DIM, typename T>
+template <int DIM>
 __global__ void __launch_bounds__(EW_T)
-    k_vcycle_out(long long n, const T* __restrict__ zin, const double* __restrict__ r, T omega,
-                 const uint8_t* __restrict__ mask, double* __restrict__ out) {
+    k_vcycle_out(long long n, const float* __restrict__ zin, const double* __restrict__ r,
+                 float omega, const uint8_t* __restrict__ mask, double* __restrict__ out) {
   const long long q0 = (long long)blockIdx.x * EW_T * EW_U + threadIdx.x;
   pdl_wait();
-  T zv[EW_U];
+  float zv[EW_U];
   bool fx[EW_U];
 #pragma unroll
   for (int u = 0; u < EW_U; ++u) {
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(EW_T)
     const long long q = q0 + u * EW_T;
     if (q >= n) continue;
     if (fx[u]) {
-      const T b = (T)r[q], z = omega * b;
+      const float b = (float)r[q], z = omega * b;
       zv[u] = z + omega * (b - z);
     }
     out[q] = (double)zv[u];
@@ -481,17 +481,14 @@ cudaError_t launch_presmooth(int t, int tin, long long n, const void* bin, void*
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_vcycle_out(int dim, int t, long long n, const void* zin, const double* r,
-                              double omega, const uint8_t* mask, double* out, cudaStream_t s) {
-  const dim3 grid(nblocks(n, EW_T * EW_U)), th(EW_T);
+cudaError_t launch_vcycle_out(int dim, long long n, const float* zin, const double* r, double omega,
+                              const uint8_t* mask, double* out, cudaStream_t s) {
   if (!zin)
     return launch_pdl(dim == 2 ? k_vcycle_fixed<2> : k_vcycle_fixed<3>,
-                      dim3(nblocks(n / dim, EW_T * 4)), th, 0, s, n / dim, r, omega, mask, out);
-  if (t == T_F64)
-    return launch_pdl(dim == 2 ? k_vcycle_out<2, double> : k_vcycle_out<3, double>, grid, th, 0, s,
-                      n, (const double*)zin, r, omega, mask, out);
-  return launch_pdl(dim == 2 ? k_vcycle_out<2, float> : k_vcycle_out<3, float>, grid, th, 0, s, n,
-                    (const float*)zin, r, (float)omega, mask, out);
+                      dim3(nblocks(n / dim, EW_T * 4)), dim3(EW_T), 0, s, n / dim, r, omega, mask,
+                      out);
+  return launch_pdl(dim == 2 ? k_vcycle_out<2> : k_vcycle_out<3>, dim3(nblocks(n, EW_T * EW_U)),
+                    dim3(EW_T), 0, s, n, zin, r, (float)omega, mask, out);
 }
 
 cudaError_t launch_convert(int tin, int tout, long long n, const void* in, void* out,
@@ -499,16 +496,14 @@ cudaError_t launch_convert(int tin, int tout, long long n, const void* in, void*
   const int nb = nblocks(n, EW_T * EW_U);
   if (tin == T_D2 && tout == T_F32)
     k_convert<float2, float><<<nb, EW_T, 0, s>>>(n, (const float2*)in, (float*)out);
-  else if (tin == T_F32 && tout == T_D2)
-    k_convert<float, float2><<<nb, EW_T, 0, s>>>(n, (const float*)in, (float2*)out);
   else if (tin == T_F64 && tout == T_F32)
     k_convert<double, float><<<nb, EW_T, 0, s>>>(n, (const double*)in, (float*)out);
   else if (tin == T_F32 && tout == T_F64)
     k_convert<float, double><<<nb, EW_T, 0, s>>>(n, (const float*)in, (double*)out);
-  else if (tin == T_F64)
+  else if (tin == T_F64 && tout == T_F64)
     k_convert<double, double><<<nb, EW_T, 0, s>>>(n, (const double*)in, (double*)out);
   else
-    k_convert<float, float><<<nb, EW_T, 0, s>>>(n, (const float*)in, (float*)out);
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 

@@ -1163,8 +1163,8 @@ to_status to_vcycle(to_ctx* c, const double* r, double* z) {
   else
     st = vcycle(c, nullptr, t, c->mixed ? l0.z2 : (void*)z, t, true);
   if (st != TO_OK) return st;
-  LAUNCH(c, launch_vcycle_out(c->dim, t, c->n, c->mixed ? l0.z2 : nullptr, r, 0.6, l0.mask, z, s),
-         "V-cycle result");
+  LAUNCH(c, launch_vcycle_out(c->dim, c->n, c->mixed ? static_cast<const float*>(l0.z2) : nullptr, r,
+                              0.6, l0.mask, z, s), "V-cycle result");
   return TO_OK;
 }
 
