@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(256)
 // 2.0 184 / 74 us, 2.5 542 / 186 us; 64 x 32 x 32, 1.5: 10 / 8 us.  (One layer
 // staged at a time: 110 us at rmin 2.0, 24 us on small grids; 8 rows instead of
 // 4: 2 to 4 us more on small grids; weights of 0 tested at run time: float64
-// comparisons, as dear as the FMAs.)
+// comparisons, as dear as the FMAs.)  Small grids take the offset list
+// (filter3_small).
 constexpr int FLX = 32, FLY = 4, FLZ = 4;
 
 template <int R>
@@ -716,11 +717,23 @@ cudaError_t launch_delta(long long nel, const double* E, const double* Eprev, do
   return cudaGetLastError();
 }
 
+// Grids on which the offset list is the faster filter: a thread per element hides
+// its loads better than a block's staging while the chip is not full.  Offset list /
+// staged, us: density filter at 16 x 8 x 8 5.2 / 6.2 (rmin 1.5), 10.3 / 12.3 (2.5), at
+// 32 x 16 x 16 6.2 / 6.2 (1.5), 6.2 / 8.2 (2.0), 10.4 / 12.3 (2.5), at 48 x 24 x 24 6.2 /
+// 6.2, 6.2 / 8.2 and 11.7 / 12.3, at 64 x 32 x 32 8.2 / 8.2 (2.0) and 14.8 / 12.3
+// (2.5).  The transpose has two values per offset: at 16 x 8 x 8 6.2 / 7.2 (1.5), 14.6 /
+// 12.3 (2.5), at 32 x 16 x 16 6.2 / 8.2 (1.5), at 48 x 24 x 24 8.2 / 8.2.
+static bool filter3_small(const GridP& g, const StencilP& st, int mode) {
+  if (mode == 1) return st.reach == 1 && g.nel <= 8192;
+  return g.nel <= (st.d2max > 2 ? 32768 : 4096);
+}
+
 cudaError_t launch_filter(int dim, const GridP& g, const StencilP& st, int mode,
                           const double* Hs, const double* in, double* out, cudaStream_t s) {
   if (dim == 2)
     k_filter<2><<<nblocks(g.nel, 256), 256, 0, s>>>(g, st, mode, Hs, in, out);
-  else if (mode != 2 && st.reach >= 1 && st.reach <= 2) {
+  else if (mode != 2 && st.reach >= 1 && st.reach <= 2 && !filter3_small(g, st, mode)) {
     const bool sens = mode == 1;
     switch (st.d2max) {
       case 1: return run_filter3<1, 1>(g, st, sens, Hs, in, out, s);
