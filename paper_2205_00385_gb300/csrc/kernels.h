@@ -92,15 +92,16 @@ struct VFuseArgs {
 // cluster size the fused kernel launches with on this device (0: unavailable)
 int vcycle_coarse_cluster(int dim, int t, int ta);
 cudaError_t launch_vcycle_coarse(int dim, int t, int ta, const VFuseArgs& a, cudaStream_t s);
-// Float32 3D finest-grid operator, two element columns per thread with packed
-// f32x2 arithmetic (kernels_pair.cu); pair_apply_ok tells whether it applies.
 // float64 finest-grid hex8 operator with the element arithmetic in 64-bit
 // fixed point (kernels_fx.cu); its tables of the Walsh blocks wht64, false where
 // the blocks do not suit it (the float64 transform then runs, kernels_fe.cu)
 bool make_fx_blocks(const double* wht64, FxBlocks* out);
 bool fx_apply_ok(const ApplyArgs& a);
 cudaError_t launch_apply_fx(const ApplyArgs& a, cudaStream_t s);
+// caches the operator's resident-block counts for the current device
 void fx_prepare();
+// Float32 3D finest-grid operator, two element columns per thread with packed
+// f32x2 arithmetic (kernels_pair.cu); pair_apply_ok tells whether it applies.
 bool pair_apply_ok(const ApplyArgs& a);
 cudaError_t launch_apply_pair(const ApplyArgs& a, cudaStream_t s);
 // caches the pair kernel's resident-block counts for the current device
@@ -135,9 +136,8 @@ cudaError_t launch_diag(int dim, const GridP& g, const uint8_t* mask, int tc, bo
                         cudaStream_t s, const Springs& sp = Springs());
 
 // ---- multigrid transfer and Galerkin operators (kernels_mg.cu) ----
-// b_c = Pm^T r_f; when zc is not null also the coarse level's smoothing from
-// a zero guess, zc = omega * dinvc * b_c.  clean: r_f is zero on every fixed
-// DOF (the fine masks are then not read; same result)
+// b_c = Pm^T r_f, r_f zero on every fixed DOF; when zc is not null also the coarse
+// level's smoothing from a zero guess, zc = omega * dinvc * b_c
 cudaError_t launch_restrict(int dim, int t, const GridP& gf, const GridP& gc, const uint8_t* mc,
                             const void* rf, void* bc, const void* dinvc, double omega, void* zc,
                             cudaStream_t s);
@@ -189,7 +189,8 @@ cudaError_t launch_convert(int tin, int tout, long long n, const void* in, void*
 // ---- vector kernels (kernels_blas.cu) ----
 cudaError_t launch_dot(long long n, const double* a, const double* b, double* partials,
                        unsigned* counter, double* out, cudaStream_t s);
-// alpha = scal[num] / scal[den]; x += alpha p; r -= alpha q; scal[rr] = r.r
+// alpha = scal[S_RZ1] / scal[S_PQ]; x += alpha p; r -= alpha q; scal[S_RR] = r.r, which
+// with the count of updates also goes to host_rr; scal[S_RZ0] = scal[S_RZ1]
 cudaError_t launch_cg_xr(long long n, double* x, double* r, const double* p, const double* q,
                          double* scal, double* partials, unsigned* counter, cudaStream_t s,
                          double* host_rr);

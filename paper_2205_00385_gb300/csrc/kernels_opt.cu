@@ -1,7 +1,8 @@
 // Design-side kernels: SIMP modulus (Eq. 1), density filter and its
 // transpose (Eq. 31-33), compliance and sensitivity (Eq. 3, 6, 34) and the
-// optimality-criteria update with a device-side bisection for the volume
-// multiplier.  All float64.
+// optimality-criteria update with a device-side search for the volume
+// multiplier.  float64, but for the mixed path's 3D sensitivity and the search,
+// which sum in double-float.
 #include <math.h>
 
 #include <algorithm>

@@ -119,10 +119,11 @@ enum Slot {
   S_RR = 0, S_PQ = 1, S_RZ0 = 2, S_RZ1 = 3, S_NRM = 4, S_TMP = 5, S_COMPL = 6,
   S_OC_L1 = 7, S_OC_L2 = 8, S_OC_VOL = 9, S_OC_DONE = 10, S_CHANGE = 11, S_EPS = 12,
   S_NRM0 = 13, S_NRM1 = 14, S_FNORM2 = 15, S_FLAG = 16,
-  // OC search: volumes and factors lambda^-eta at the bracket's ends, the
-  // sweep's multipliers and their factors
   S_CG_COUNT = 21,   // updates of the current solve
-  S_OC_V1 = 17, S_OC_V2 = 18, S_OC_S1 = 19, S_OC_S2 = 20, S_OC_NPT = 8, S_OC_PT = 24, S_OC_SP = S_OC_PT + S_OC_NPT,
+  // OC search: volumes and factors lambda^-eta at the bracket's ends, the
+  // sweep's multipliers and their factors (room for S_OC_NPT each)
+  S_OC_V1 = 17, S_OC_V2 = 18, S_OC_S1 = 19, S_OC_S2 = 20,
+  S_OC_NPT = 8, S_OC_PT = 24, S_OC_SP = S_OC_PT + S_OC_NPT,
   S_NSLOTS = 64
 };
 
