@@ -177,8 +177,8 @@ __global__ void __launch_bounds__(DX * DY)
 // rows of the four elements around it, each row a Dot2 sum.  About 950 FP32
 // instructions per node; the direction is zero on the fixed DOFs (a fixed row's
 // product is 0).  Twelve solves at 640 x 320 to 1e-6: 1001 iterations in 129 ms
-// with the float32 product, 738 in 76 ms with this one (float64: 726); at
-// 320 x 160 614 in 67 ms and 307 in 25 ms.
+// with the float32 product, 730 in 74 ms with this one (float64: 726); at
+// 320 x 160 614 in 67 ms and 307 in 24 ms.
 // ---------------------------------------------------------------------------
 struct DfKe2 {
   float2 v[8][8];
