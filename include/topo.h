@@ -367,7 +367,10 @@ to_status to_filter(to_ctx* ctx, int32_t mode, const double* in, double* out);
  * min(1, rho+move)) with lam searched on [0, 1e9] to a relative
  * bracket of 1e-13 so that sum_e dv_f,e rho_new,e = volfrac*nel (the
  * filtered volume when dv_f = H^T(1/Hs), Eq. 3).  dc_f, dv_f: dev nel.
- * change_dev (dev, 1 double, may be NULL): max |rho_new - rho|. */
+ * change_dev (dev, 1 double, may be NULL): max |rho_new - rho|.  Nothing waits for
+ * the host; a search that goes on after its first sweeps runs as blocks that wait for
+ * each other, and if such a wait should ever expire (seconds) the next solve returns
+ * TO_E_TIMEOUT. */
 to_status to_oc_update(to_ctx* ctx, double volfrac, double move, const double* dc_f,
                        const double* dv_f, double* rho, double* change_dev);
 

@@ -149,7 +149,8 @@ __host__ __device__ __forceinline__ void fx_element(const FxBlocks& kb, double c
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const int s = ec[c] - e, l = s > 0 ? s : 0, r = s < 0 ? -s : 0;
+    // (a component without modes is zero, whatever its shift)
+    const int s = ec[c] - e, l = s > 0 ? (s < 63 ? s : 63) : 0, r = s < 0 ? -s : 0;
 #pragma unroll
     for (int t = 1; t < 8; ++t) X[c][t] = fx_shr((fx_t)((unsigned long long)X[c][t] << l), r);
   }
